@@ -600,11 +600,14 @@ static void dense_lu(double *a, int *piv, int n) {
 
 static void dense_lu_solve(const double *a, const int *piv, int n, const double *b, double *x) {
   for (int i = 0; i < n; ++i) x[i] = b[i];
+  /* dense_lu exchanges whole rows, the multipliers in them too: every
+   * exchange comes before the first elimination */
   for (int k = 0; k < n; ++k) {
     int p = piv[k];
     if (p != k) { double t = x[k]; x[k] = x[p]; x[p] = t; }
-    for (int i = k + 1; i < n; ++i) x[i] -= a[(size_t)i * n + k] * x[k];
   }
+  for (int k = 0; k < n; ++k)
+    for (int i = k + 1; i < n; ++i) x[i] -= a[(size_t)i * n + k] * x[k];
   for (int i = n - 1; i >= 0; --i) {
     double s = x[i];
     for (int j = i + 1; j < n; ++j) s -= a[(size_t)i * n + j] * x[j];

@@ -174,12 +174,13 @@ __device__ void dense_solve_cta(int n, const double *a, const int *piv, const T 
   int t = threadIdx.x, nt = blockDim.x;
   for (int i = t; i < n; i += nt) xs[i] = double(__ldcg(b + i));
   __syncthreads();
-  for (int k = 0; k < n; ++k) {
-    if (t == 0) {
+  if (t == 0)   // every row exchange first (see k_dense_solve)
+    for (int k = 0; k < n; ++k) {
       int p = piv[k];
       if (p != k && p >= 0 && p < n) { double tmp = xs[k]; xs[k] = xs[p]; xs[p] = tmp; }
     }
-    __syncthreads();
+  __syncthreads();
+  for (int k = 0; k < n; ++k) {
     double xk = xs[k];
     for (int i = k + 1 + t; i < n; i += nt) xs[i] -= a[(size_t)i * n + k] * xk;
     __syncthreads();

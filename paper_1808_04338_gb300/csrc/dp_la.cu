@@ -1138,12 +1138,15 @@ __global__ void __launch_bounds__(1024) k_dense_solve(int n, const double *a, co
   int t = threadIdx.x, nt = blockDim.x;
   for (int i = t; i < n; i += nt) xs[i] = double(b[i]);
   __syncthreads();
-  for (int k = 0; k < n; ++k) {
-    if (t == 0) {
+  // k_dense_lu exchanges whole rows, the multipliers in them too: every
+  // exchange comes before the first elimination
+  if (t == 0)
+    for (int k = 0; k < n; ++k) {
       int p = piv[k];
       if (p != k && p >= 0 && p < n) { double tmp = xs[k]; xs[k] = xs[p]; xs[p] = tmp; }
     }
-    __syncthreads();
+  __syncthreads();
+  for (int k = 0; k < n; ++k) {
     double xk = xs[k];
     for (int i = k + 1 + t; i < n; i += nt) xs[i] -= a[(size_t)i * n + k] * xk;
     __syncthreads();
@@ -1172,6 +1175,8 @@ __global__ void k_dense_inverse(int n, const double *a, const int *piv, double *
       inv[(size_t)k * n + c] = inv[(size_t)p * n + c];
       inv[(size_t)p * n + c] = tmp;
     }
+  }
+  for (int k = 0; k < n; ++k) {
     double xk = inv[(size_t)k * n + c];
     for (int i = k + 1; i < n; ++i) inv[(size_t)i * n + c] -= a[(size_t)i * n + k] * xk;
   }
