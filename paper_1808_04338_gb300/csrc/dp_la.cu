@@ -1189,6 +1189,172 @@ __global__ void k_dense_inverse(int n, const double *a, const int *piv, double *
 }
 
 
+// The usual coarsest operator (at most kFactorMax rows; the default
+// hierarchy stops at 128): LU with partial pivoting in one CTA's shared
+// memory, straight from the level's CSR, then the inverse's columns in
+// parallel over the GPU (k_dense_cols).  Before, the dense copy, the LU and
+// the inverse each walked global memory, the inverse a column a thread in
+// one CTA: a chain of L2 round trips (146 + 146 us at 36 rows, 430 + 990 us
+// at 91).  Bound now by the chain of pivots for small n and by the SM's two
+// FP64 FMAs a cycle from about 60 rows on (n^3 / 3 of them).
+//
+// Rows are not moved: order[i] is the step that took row i as its pivot.
+// In step k warp 0 updates column k + 1 first, picks its pivot (largest
+// magnitude, NaN never, the first free row when there is none) and forms its
+// multipliers, while the other warps update columns k + 2 on: one barrier a
+// step.  Output: lu column-major in pivot order (leading dimension ldo, even,
+// so that the columns can be read as 16-byte words), prow[k] the row of
+// pivot k, rdiag[k] its reciprocal (0 for a zero pivot, whose multipliers
+// are then 0 as well).
+constexpr int kFactorMax = 160, kFactorThreads = 512;
+inline int factor_ld(int n) { return (n + 1) & ~1; }
+inline size_t factor_smem(int n) { return ((size_t)n * (n | 1) + 2 * (size_t)n) * 8; }
+
+__global__ void __launch_bounds__(kFactorThreads) k_dense_factor(int n, const int *rowptr,
+                                                                 const int *col,
+                                                                 const double *val, double *lu,
+                                                                 int ldo, int *prow,
+                                                                 double *rdiag) {
+  extern __shared__ double fac[];
+  __shared__ int piv[kFactorMax], order[kFactorMax];
+  const int ld = n | 1, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int kWarps = kFactorThreads / 32;
+  double *A = fac, *mult = fac + (size_t)n * ld;   // mult: by the step's parity
+  for (int q = threadIdx.x; q < n * ld; q += kFactorThreads) A[q] = 0.0;
+  for (int i = threadIdx.x; i < n; i += kFactorThreads) order[i] = n;
+  __syncthreads();
+  for (int i = warp; i < n; i += kWarps)
+    for (int e = rowptr[i] + lane, e1 = rowptr[i + 1]; e < e1; e += 32) A[i * ld + col[e]] = val[e];
+  __syncthreads();
+  // warp 0: the pivot of column k and its multipliers
+  auto panel = [&](int k) {
+    unsigned long long best = 0;   // |a| as its bits + 1, 0: no candidate
+    int bi = n;
+    for (int i = lane; i < n; i += 32) {
+      if (order[i] < n) continue;
+      unsigned long long b = (unsigned long long)__double_as_longlong(A[i * ld + k]) &
+                             0x7fffffffffffffffull;
+      b = b > 0x7ff0000000000000ull ? 0 : b + 1;
+      if (bi == n || b > best) { best = b; bi = i; }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
+      int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (oi < n && (bi == n || ob > best || (ob == best && oi < bi))) { best = ob; bi = oi; }
+    }
+    double d = A[bi * ld + k], r = d != 0.0 ? 1.0 / d : 0.0;
+    __syncwarp();
+    if (lane == 0) {
+      order[bi] = k;
+      piv[k] = bi;
+      prow[k] = bi;
+      rdiag[k] = r;
+    }
+    __syncwarp();
+    for (int i = lane; i < n; i += 32)
+      if (order[i] == n) {
+        double l = d != 0.0 ? A[i * ld + k] / d : 0.0;
+        A[i * ld + k] = l;
+        mult[(k & 1) * n + i] = l;
+      }
+    __syncwarp();
+  };
+  if (warp == 0) panel(0);
+  __syncthreads();
+  for (int k = 0; k + 1 < n; ++k) {
+    const double *u = A + piv[k] * ld, *l = mult + (k & 1) * n;
+    if (warp == 0) {
+      double uk = u[k + 1];
+      for (int i = lane; i < n; i += 32)
+        if (order[i] == n) A[i * ld + k + 1] -= l[i] * uk;
+      __syncwarp();
+      panel(k + 1);
+    } else {
+      for (int i = warp - 1; i < n; i += kWarps - 1) {
+        if (order[i] <= k) continue;   // the pivot of step k + 1 may be marked meanwhile
+        double li = l[i];
+        for (int j = k + 2 + lane; j < n; j += 32) A[i * ld + j] -= li * u[j];
+      }
+    }
+    __syncthreads();
+  }
+  for (int j = warp; j < n; j += kWarps)
+    for (int k = lane; k < n; k += 32) lu[(size_t)j * ldo + k] = A[piv[k] * ld + j];
+}
+
+// Columns of the inverse from k_dense_factor's output, a warp per column
+// (two per CTA, over the GPU): the two substitutions with the column in
+// registers (R = ceil(n / 32) values a lane), the factors in shared memory.
+template <int R>
+__global__ void __launch_bounds__(64) k_dense_cols(int n, const double *__restrict__ lu, int ldo,
+                                                   const int *__restrict__ prow,
+                                                   const double *__restrict__ rdiag, double *inv) {
+  extern __shared__ double fac[];
+  const double2 *src = reinterpret_cast<const double2 *>(lu);
+  double2 *dst = reinterpret_cast<double2 *>(fac);
+  int tot = n * ldo / 2;
+#pragma unroll 8
+  for (int q = threadIdx.x; q < tot; q += 64) dst[q] = __ldg(src + q);
+  __syncthreads();
+  const int lane = threadIdx.x & 31, c = 2 * blockIdx.x + (threadIdx.x >> 5);
+  if (c >= n) return;   // whole warps
+  double x[R], rd[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    int i = lane + 32 * r;
+    x[r] = i < n && __ldg(prow + i) == c ? 1.0 : 0.0;
+    rd[r] = i < n ? __ldg(rdiag + i) : 0.0;
+  }
+#pragma unroll
+  for (int b = 0; b < R; ++b)
+#pragma unroll 4
+    for (int kk = 0; kk < 32; ++kk) {
+      int k = 32 * b + kk;
+      if (k >= n) break;
+      double xk = __shfl_sync(0xffffffffu, x[b], kk);
+      const double *l = fac + (size_t)k * ldo;
+#pragma unroll
+      for (int r = b; r < R; ++r) {
+        int i = lane + 32 * r;
+        if (i > k && i < n) x[r] -= l[i] * xk;
+      }
+    }
+#pragma unroll
+  for (int b = R - 1; b >= 0; --b)
+#pragma unroll 4
+    for (int kk = 31; kk >= 0; --kk) {
+      int k = 32 * b + kk;
+      if (k >= n) continue;
+      double xk = __shfl_sync(0xffffffffu, x[b] * rd[b], kk);
+      if (lane == kk) x[b] = xk;
+      const double *u = fac + (size_t)k * ldo;
+#pragma unroll
+      for (int r = 0; r <= b; ++r) {
+        int i = lane + 32 * r;
+        if (i < k) x[r] -= u[i] * xk;
+      }
+    }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    int i = lane + 32 * r;
+    if (i < n) inv[(size_t)i * n + c] = x[r];
+  }
+}
+
+template <int R>
+static void dense_cols(Sim *s, int n) {
+  static const bool once = [] {
+    cudaFuncSetAttribute(k_dense_cols<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         kFactorMax * kFactorMax * 8);
+    return true;
+  }();
+  (void)once;
+  int ldo = factor_ld(n);
+  DP_LAUNCH(s, k_dense_cols<R>, nblk(n, 2), 64, (size_t)n * ldo * 8, n, s->coarse_lu, ldo,
+            s->coarse_piv, s->coarse_lu + (size_t)n * ldo, s->coarse_inv);
+}
+
 int coarse_factor(Sim *s) {
   Level &L = s->lev.back();
   int n = L.n;
@@ -1196,7 +1362,8 @@ int coarse_factor(Sim *s) {
   if (!s->coarse_lu || s->coarse_n != n) {
     if (s->coarse_lu) dfree(s, s->coarse_lu);
     if (s->coarse_piv) dfree(s, s->coarse_piv);
-    s->coarse_lu = (double *)dalloc(s, (size_t)n * n * 8);
+    // the factors, and after k_dense_factor's the pivots' reciprocals
+    s->coarse_lu = (double *)dalloc(s, (size_t)n * (factor_ld(n) + 1) * 8);
     s->coarse_piv = (int *)dalloc(s, (size_t)n * 4);
     if (!s->coarse_lu || !s->coarse_piv) { s->fail(DP_ENOMEM, "allocation failed"); return DP_ENOMEM; }
     if (s->coarse_inv) dfree(s, s->coarse_inv);
@@ -1207,6 +1374,26 @@ int coarse_factor(Sim *s) {
     }
   }
   s->coarse_n = n;
+  if (n <= kFactorMax) {
+    static const bool once = [] {
+      cudaFuncSetAttribute(k_dense_factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)factor_smem(kFactorMax));
+      return true;
+    }();
+    (void)once;
+    int ldo = factor_ld(n);
+    DP_LAUNCH(s, k_dense_factor, 1, kFactorThreads, factor_smem(n), n, L.rowptr, L.col, L.val,
+              s->coarse_lu, ldo, s->coarse_piv, s->coarse_lu + (size_t)n * ldo);
+    switch ((n + 31) / 32) {
+      case 1: dense_cols<1>(s, n); break;
+      case 2: dense_cols<2>(s, n); break;
+      case 3: dense_cols<3>(s, n); break;
+      case 4: dense_cols<4>(s, n); break;
+      default: dense_cols<5>(s, n); break;
+    }
+    DP_CUDA(s, cudaGetLastError());
+    return DP_OK;
+  }
   DP_LAUNCH(s, k_csr_to_dense, nblk(n), kBlock, 0, n, L.rowptr, L.col, L.val, s->coarse_lu);
   DP_LAUNCH(s, k_dense_lu, 1, 1024, 0, n, s->coarse_lu, s->coarse_piv);
   if (s->coarse_inv)
