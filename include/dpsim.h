@@ -141,9 +141,10 @@ typedef struct {
   int32_t amg_gs_levels;
   int32_t cluster_rows;  /* AMG levels of at most this many rows run inside one
                             thread-block-cluster launch per V-cycle (with
-                            use_graphs); < 0: never; 0: the library default,
-                            20000 rows when one of those levels uses
-                            Gauss-Seidel, else never */
+                            use_graphs), from the first of them whose vectors fit
+                            in the cluster's shared memory; < 0: never; 0: the
+                            library default, 20000 rows when one of those levels
+                            uses Gauss-Seidel, else never */
   int32_t amg_refresh;   /* 0: the prolongators and coarse operators are recomputed
                             every Newton iteration; 1: only at the first Newton
                             iteration of a timestep (level 0, the pressure block,

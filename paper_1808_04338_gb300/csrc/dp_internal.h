@@ -71,10 +71,12 @@ struct Level {
   int *colour = nullptr, ncolour = 0;
   int *clist = nullptr;                  // rows sorted by (colour, index)
   std::vector<int> cstart;               // host: colour c rows clist[cstart[c]..cstart[c+1])
-  int *cstart_dev = nullptr;             // the same on the device
-  int *ell_col = nullptr, *ell_src = nullptr, *ell_off = nullptr, *ell_K = nullptr;
-  double *ell_val = nullptr;             // padded per-colour copy (cluster cycle)
+  int *ell_col = nullptr, *ell_src = nullptr;   // padded per-colour copy (cluster cycle)
+  double *ell_val = nullptr;
   float *ell_valf = nullptr;
+  double *ell_dinv = nullptr;            // 1 / a_ii by row slot of the padded copy
+  float *ell_dinvf = nullptr;
+  int *ell_desc = nullptr;               // per colour: first slot, rows, offset, shape
   long long ell_total = 0;
   double *fdiag = nullptr, *ratio = nullptr;
   // prolongator P (n x nagg), restriction R = P^T (nagg x n), AP = A P
@@ -258,7 +260,7 @@ int autotune(Sim *s, int reps, std::string &report);
 // dp_cycle.cu (the coarse levels of the V-cycle in one cluster launch)
 constexpr int kClusterMaxRows = 20000;   // default of dp_options.cluster_rows
 int cluster_setup(Sim *s);
-int cluster_refresh(Sim *s);
+int cluster_refresh(Sim *s, bool coarse);
 template <typename T> int coarse_cycle(Sim *s, int l0, const T *b, T *x);
 
 struct Timing {
@@ -386,7 +388,10 @@ struct Sim {
   int *coarse_piv = nullptr;
   int coarse_n = 0;
   int cl_level = -1, cl_size = 0;                    // first level of the cluster cycle
-  void *cl_lev64 = nullptr, *cl_lev32 = nullptr;     // device level descriptors
+  void *cl_lev = nullptr;                            // device level descriptors
+  int cl_smem = 0, cl_dense = 0;                     // shared bytes of a CTA of the cycle, and
+  bool cl_rep = false;                               //   where its dense solve's vector starts;
+                                                     //   b and r replicated too
   double *omega = nullptr;                           // device scalars
   unsigned long long *rho_bits = nullptr;
   int *counter = nullptr, *h_counter = nullptr;      // device / pinned host

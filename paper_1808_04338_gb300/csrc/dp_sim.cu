@@ -489,7 +489,7 @@ int solve_prepare(Sim *s, double *eta, bool norms_current) {
     else DP_TRY(level_dinv(s, s->lev[0]));   // level 0 only: its values are s->ap
     if (s->opt.precision >= 1) DP_TRY(mixed_refresh(s, coarse));
     DP_TRY(l0_refresh(s, coarse));
-    if (coarse) DP_TRY(cluster_refresh(s));
+    DP_TRY(cluster_refresh(s, coarse));
   }
   return DP_OK;
 }

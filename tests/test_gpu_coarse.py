@@ -39,3 +39,25 @@ def test_dense_coarsest_level(nx, wells):
     prob = small(nx, 1, 1, wells=wells)
     g, o = relres(prob, 2, interior(prob, nx), amg_coarse_max=256)
     assert abs(g - o) <= 1e-6 * o + 1e-12
+
+
+# where the cluster cycle's vectors live (FP64, shared budget 224 KB): everything
+# replicated (levels of 3268 rows down); x replicated, the right-hand sides and
+# residuals in global memory (about 15000 rows down, its colours in several
+# trips); a level whose x does not fit (29828 rows) is left to its own launches;
+# l1-Jacobi below the finest in the cluster
+@pytest.mark.parametrize("grid,gs_levels,cluster_rows",
+                         [((100, 100, 10), 30, 4000), ((80, 80, 8), 30, 0),
+                          ((100, 100, 10), 30, 40000), ((80, 80, 8), 1, 20000)])
+def test_cluster_cycle_vectors(grid, gs_levels, cluster_rows):
+    g, o = relres(di.layered(*grid), 3, amg_gs_levels=gs_levels, cluster_rows=cluster_rows)
+    assert abs(g - o) <= 1e-6 * o
+
+
+@pytest.mark.parametrize("coarse_max", [2, 40, 2000])
+def test_cluster_cycle_from_level_0(coarse_max):
+    """The whole cycle in the cluster (602 rows), down to a coarsest level that
+    is smoothed, dense, or level 0 itself."""
+    prob = di.tiny()
+    g, o = relres(prob, 3, interior(prob, 5), amg_coarse_max=coarse_max)
+    assert abs(g - o) <= 1e-6 * o + 1e-12
