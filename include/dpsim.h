@@ -188,7 +188,8 @@ typedef struct dp_sim dp_sim;
  * DPSIM_PDL, read once per process, is a bit mask of the classes to launch
  * that way (1 level-0 well rows, 2 the V-cycle below level 0, 4 the latter
  * letting their own dependents in early, 8 level 0's colour kernels, 16 the
- * ILU(0) forward well rows; default 31, all); results do not depend on it. */
+ * ILU(0) forward well rows, 32 every other kernel of an Arnoldi step in small
+ * and mid-size realisations; default 63, all); results do not depend on it. */
 
 /* Create a realisation: copies grid, rock, fluid and wells, computes the
  * well indices (Peaceman's radius for a vertical well, Section 2), builds

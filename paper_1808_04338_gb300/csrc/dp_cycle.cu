@@ -414,7 +414,7 @@ template <typename T, bool REP>
 __global__ void __launch_bounds__(kClusterThreads, 1)
     k_coarse_cycle(const LevelDev<T> *__restrict__ lv, int l0, int nl, const T *b0, T *x0,
                    const double *lu, const int *piv, const double *inv, int dense_n,
-                   int dense_smem) {
+                   int dense_smem, int trig) {
   extern __shared__ __align__(16) unsigned char cyc_smem[];
   T *sm = reinterpret_cast<T *>(cyc_smem);
   using VB = typename Side<T, REP>::t;
@@ -430,6 +430,8 @@ __global__ void __launch_bounds__(kClusterThreads, 1)
     if constexpr (REP) return VB{sm + lv[l].ro};
     else return VB{lv[l].r};
   };
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   for (int l = l0; l < nl; ++l) {
     if (lv[l].l1) continue;   // an l1-Jacobi level writes its x whole
     T *x = sm + lv[l].xo;
@@ -701,9 +703,9 @@ int cluster_refresh(Sim *s, bool coarse) {
 static int cluster_ctas() {
   static const int ctas = [] {
     using Cycle64 = void (*)(const LevelDev<double> *, int, int, const double *, double *,
-                             const double *, const int *, const double *, int, int);
+                             const double *, const int *, const double *, int, int, int);
     using Cycle32 = void (*)(const LevelDev<float> *, int, int, const float *, float *,
-                             const double *, const int *, const double *, int, int);
+                             const double *, const int *, const double *, int, int, int);
     const Cycle64 k64[2] = {k_coarse_cycle<double, false>, k_coarse_cycle<double, true>};
     const Cycle32 k32[2] = {k_coarse_cycle<float, false>, k_coarse_cycle<float, true>};
     for (int k = 0; k < 2; ++k) {
@@ -792,11 +794,14 @@ int coarse_cycle(Sim *s, int l0, const T *b, T *x) {
   cfg.blockDim = dim3(kClusterThreads);
   cfg.dynamicSmemBytes = s->cl_smem;
   cfg.stream = s->stream;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = s->cl_size; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  const bool pdl = s->pdl_small && (pdl_mode() & kPdlSmall);
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = pdl ? 2 : 1;
   const LevelDev<T> *lv = (const LevelDev<T> *)s->cl_lev;
   int nl = (int)s->lev.size();
   {
@@ -804,7 +809,7 @@ int coarse_cycle(Sim *s, int l0, const T *b, T *x) {
     DP_CUDA(s, cudaLaunchKernelEx(&cfg, s->cl_rep ? k_coarse_cycle<T, true> : k_coarse_cycle<T, false>,
                                   lv, l0, nl, b, x, (const double *)s->coarse_lu,
                                   (const int *)s->coarse_piv, (const double *)s->coarse_inv,
-                                  s->coarse_n, s->cl_dense));
+                                  s->coarse_n, s->cl_dense, pdl && pdl_trigger() ? 1 : 0));
   }
   return DP_OK;
 }

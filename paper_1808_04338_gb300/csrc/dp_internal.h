@@ -147,14 +147,20 @@ struct RegionScope {
 // it (launch_pdl, after Sim).  cls: kPdlWells, the level-0 well rows;
 // kPdlCoarse, the kernels of the V-cycle's transfers and coarse levels;
 // kPdlL0, level 0's pipelined colour kernels (Gauss-Seidel and residual);
-// kPdlIluW, the ILU(0) forward sweep's long rows (the wells).
+// kPdlIluW, the ILU(0) forward sweep's long rows (the wells); kPdlSmall, all
+// other kernels of an Arnoldi step, in realisations of at most kPdlSmallRows
+// block rows (Sim::pdl_small).
 #define DP_LAUNCH_PDL(sim, cls, name, grid, block, smem, ...)                         \
   do {                                                                               \
     if ((sim)->alloc_failed) break;                                                  \
     ::dp::LaunchScope ls__((sim), #name);                                            \
     ::dp::launch_pdl((sim), (cls), name, dim3(grid), dim3(block), (smem), __VA_ARGS__); \
   } while (0)
-constexpr int kPdlWells = 1, kPdlCoarse = 2, kPdlL0 = 8, kPdlIluW = 16;
+constexpr int kPdlWells = 1, kPdlCoarse = 2, kPdlL0 = 8, kPdlIluW = 16, kPdlSmall = 32;
+// Where kernels are short a launch's placement shows: a 602-row timestep 8.6
+// -> 8.2 ms, Example 2's run 34.5 -> 33.7 ms; from about 200k rows the early
+// CTAs cost as much as they save (96.2 -> 98.4 and 17.7 -> 17.9 ms).
+constexpr int kPdlSmallRows = 65536;
 // Waits until the grids this one depends on have completed and their
 // writes are visible (a no-op in a kernel launched without the attribute).
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -402,6 +408,7 @@ struct Sim {
   double *dots_part = nullptr, *dots = nullptr, *scal = nullptr;
   double *h_res = nullptr;                           // pinned host scalars
   int dot_blocks = 0;
+  bool pdl_small = false;   // kPdlSmall applies (see kPdlSmallRows)
   double *z1 = nullptr, *r1 = nullptr, *rp = nullptr, *xp = nullptr;
   // CUDA graphs of the FGMRES iterations j = 0..m-1 (captured on first use)
   std::vector<cudaGraphExec_t> graph;
@@ -443,7 +450,7 @@ inline void launch_pdl(Sim *s, int cls, void (*k)(P...), dim3 grid, dim3 block, 
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = (pdl_mode() & cls) ? 1 : 0;
+  cfg.numAttrs = (pdl_mode() & cls) && (cls != kPdlSmall || s->pdl_small) ? 1 : 0;
   cudaError_t e = cudaLaunchKernelEx(&cfg, k, std::forward<A>(args)...);
   if (e != cudaSuccess) s->fail(DP_ECUDA, std::string("kernel launch: ") + cudaGetErrorString(e));
 }

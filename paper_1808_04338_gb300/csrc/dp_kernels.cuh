@@ -338,7 +338,7 @@ __device__ __forceinline__ void k_bsr_resid_f32_b(int bx, int gx, int n, int nL,
 // The start of level 0's pre-smoothing fused into the kernel that writes
 // its right-hand side (level 0 in colour order, the sweep starting from x =
 // 0): with x set, every row's x is written as well, b/a_ii (the reduced
-// Gauss-Seidel formula, as in k_gs_c_first) on the first colour's rows
+// Gauss-Seidel formula, as in k_gs_c_start) on the first colour's rows
 // [f0, f1), 0 on the others.
 struct X0Init {
   float *x = nullptr;

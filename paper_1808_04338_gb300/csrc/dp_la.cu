@@ -41,7 +41,9 @@ __global__ void __launch_bounds__(kBlock) k_bsr_spmv(int n, int nL, int nc, int 
                                                      const double *__restrict__ val,
                                                      const double *__restrict__ x,
                                                      const double *__restrict__ b,
-                                                     double *__restrict__ y) {
+                                                     double *__restrict__ y, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   k_bsr_spmv_b<MODE>(blockIdx.x, gridDim.x, n, nL, nc, nlong, rowptr, col, val, x, b, y);
 }
 
@@ -118,7 +120,9 @@ __global__ void __launch_bounds__(kBlock) k_bsr_presid(int n, int nL, int nc, in
                                                        const double *__restrict__ x,
                                                        const double *__restrict__ b,
                                                        double *__restrict__ rp,
-                                                       const int *__restrict__ omap) {
+                                                       const int *__restrict__ omap, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   if (blockIdx.x == 0) {   // the well rows, a warp per row (as in k_bsr_spmv)
     int lane = threadIdx.x & 31;
     const double2 *x2 = reinterpret_cast<const double2 *>(x);
@@ -171,7 +175,9 @@ __global__ void __launch_bounds__(kBlock) k_bsr_resid_f32(int n, int nL, int nc,
                                                          const float *__restrict__ valf,
                                                          const float *__restrict__ x,
                                                          const double *__restrict__ b,
-                                                         float *__restrict__ y) {
+                                                         float *__restrict__ y, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   k_bsr_resid_f32_b(blockIdx.x, gridDim.x, n, nL, nc, nlong, rowptr, col, valf, x, b, y);
 }
 
@@ -185,21 +191,27 @@ __global__ void __launch_bounds__(kBlock) k_bsr_presid_f32(int n, int nL, int nc
                                                           const double *__restrict__ b,
                                                           float *__restrict__ rp,
                                                           const int *__restrict__ omap,
-                                                          X0Init xi) {
+                                                          X0Init xi, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   k_bsr_presid_f32_b(blockIdx.x, gridDim.x, n, nL, nc, nlong, rowptr, col, pf, x, b, rp, omap, xi);
 }
 
+// A kernel of class kPdlSmall lets its own dependent in once past its wait
+// when the realisation's kernels are launched that way.
+static int small_trig(const Sim *s) { return s->pdl_small && pdl_trigger() ? 1 : 0; }
+
 int bsr_spmv(Sim *s, const double *x, double *y) {
-  DP_LAUNCH(s, k_bsr_spmv<0>, 1 + nblk(2LL * s->sv_long0), kBlock, 0, s->K.n, s->sv_sL, s->sv_sc,
+  DP_LAUNCH_PDL(s, kPdlSmall, k_bsr_spmv<0>, 1 + nblk(2LL * s->sv_long0), kBlock, 0, s->K.n, s->sv_sL, s->sv_sc,
             s->sv_long0,
-            s->srowptr, s->scol, s->sval, x, nullptr, y);
+            s->srowptr, s->scol, s->sval, x, nullptr, y, small_trig(s));
   return DP_OK;
 }
 
 int bsr_residual(Sim *s, const double *b, const double *x, double *r) {
-  DP_LAUNCH(s, k_bsr_spmv<1>, 1 + nblk(2LL * s->sv_long0), kBlock, 0, s->K.n, s->sv_sL, s->sv_sc,
+  DP_LAUNCH_PDL(s, kPdlSmall, k_bsr_spmv<1>, 1 + nblk(2LL * s->sv_long0), kBlock, 0, s->K.n, s->sv_sL, s->sv_sc,
             s->sv_long0,
-            s->srowptr, s->scol, s->sval, x, b, r);
+            s->srowptr, s->scol, s->sval, x, b, r, small_trig(s));
   return DP_OK;
 }
 
@@ -339,6 +351,7 @@ __global__ void __launch_bounds__(kBlock) k_ilu_fwd(int r0, int r1, const int *_
                                                     const T *__restrict__ lu,
                                                     const TR *__restrict__ rhs, T *zp) {
   griddep_launch_dependents();   // the long rows after this colour (k_ilu_fwd_wp)
+  griddep_wait();
   k_ilu_fwd_b<T, TR>(blockIdx.x, gridDim.x, r0, r1, perm, Lptr, colp, lu, rhs, zp);
 }
 
@@ -368,7 +381,9 @@ __global__ void __launch_bounds__(kBlock, kTailMinBlocks) k_ilu_fwd_t(int r0, in
 // permutation loads, then their right-hand-side loads, issued together.
 template <typename T, typename TR>
 __global__ void __launch_bounds__(kBlock) k_ilu_fwd_copy(int r0, int r1, const int *__restrict__ perm,
-                                                     const TR *__restrict__ rhs, T *zp) {
+                                                     const TR *__restrict__ rhs, T *zp, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   k_ilu_fwd_copy_b<T, TR>(blockIdx.x, gridDim.x, r0, r1, perm, rhs, zp);
 }
 
@@ -382,7 +397,9 @@ template <typename T>
 __global__ void __launch_bounds__(kBlock) k_ilu_bwd_r(int r0, int r1, int nL, int n,
                                                       const int *__restrict__ Uptr,
                                                       const int *__restrict__ colp,
-                                                      const T *__restrict__ lu, T *zp) {
+                                                      const T *__restrict__ lu, T *zp, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   k_ilu_bwd_r_b<T>(blockIdx.x, gridDim.x, r0, r1, nL, n, Uptr, colp, lu, zp);
 }
 
@@ -395,7 +412,9 @@ __global__ void __launch_bounds__(kBlock) k_ilu_fwd_w(int r0, int r1, int nL,
                                                       const int *__restrict__ Lptr,
                                                       const int *__restrict__ colp,
                                                       const T *__restrict__ lu,
-                                                      const TR *__restrict__ rhs, T *zp) {
+                                                      const TR *__restrict__ rhs, T *zp, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   k_ilu_fwd_w_b<T, TR, PIVOT>(blockIdx.x, gridDim.x, r0, r1, nL, perm, Lptr, colp, lu, rhs, zp);
 }
 
@@ -403,7 +422,9 @@ template <typename T>
 __global__ void __launch_bounds__(kBlock) k_ilu_bwd_w(int r0, int r1, int nL, int n,
                                                       const int *__restrict__ Uptr,
                                                       const int *__restrict__ colp,
-                                                      const T *__restrict__ lu, T *zp) {
+                                                      const T *__restrict__ lu, T *zp, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   k_ilu_bwd_w_b<T>(blockIdx.x, gridDim.x, r0, r1, nL, n, Uptr, colp, lu, zp);
 }
 
@@ -725,16 +746,16 @@ static int ilu_apply_t(Sim *s, const T *lu, const TR *r, T *zpo = nullptr) {
         DP_LAUNCH_PDL(s, kPdlIluW, (k_ilu_fwd_wp<T, TR, false>), r1 - r0, 32, 0, r0, nL, s->perm,
                       s->lu_Lptr, s->lu_colp, lu, r, zp);
     } else if (c == last && s->lu_cmaxlen[c] > kLongRow)
-      DP_LAUNCH(s, (k_ilu_fwd_w<T, TR, true>), nblk(32LL * (r1 - r0)), kBlock, 0, r0, r1, nL,
-                s->perm, s->lu_Lptr, s->lu_colp, lu, r, zp);
+      DP_LAUNCH_PDL(s, kPdlSmall, (k_ilu_fwd_w<T, TR, true>), nblk(32LL * (r1 - r0)), kBlock, 0, r0, r1, nL,
+                s->perm, s->lu_Lptr, s->lu_colp, lu, r, zp, small_trig(s));
     else if (s->lu_cmaxlen[c] > kLongRow)
-      DP_LAUNCH(s, (k_ilu_fwd_w<T, TR, false>), nblk(32LL * (r1 - r0)), kBlock, 0, r0, r1, nL,
-                s->perm, s->lu_Lptr, s->lu_colp, lu, r, zp);
+      DP_LAUNCH_PDL(s, kPdlSmall, (k_ilu_fwd_w<T, TR, false>), nblk(32LL * (r1 - r0)), kBlock, 0, r0, r1, nL,
+                s->perm, s->lu_Lptr, s->lu_colp, lu, r, zp, small_trig(s));
     else if (c == first)   // no L blocks
-      DP_LAUNCH(s, (k_ilu_fwd_copy<T, TR>), nblk((r1 - r0 + kRes - 1) / kRes), kBlock, 0, r0, r1,
-                s->perm, r, zp);
+      DP_LAUNCH_PDL(s, kPdlSmall, (k_ilu_fwd_copy<T, TR>), nblk((r1 - r0 + kRes - 1) / kRes), kBlock, 0, r0, r1,
+                s->perm, r, zp, small_trig(s));
     else
-      DP_LAUNCH(s, (k_ilu_fwd<T, TR>), nblk(2LL * (r1 - r0)), kBlock, 0, r0, r1, s->perm,
+      DP_LAUNCH_PDL(s, kPdlSmall, (k_ilu_fwd<T, TR>), nblk(2LL * (r1 - r0)), kBlock, 0, r0, r1, s->perm,
                 s->lu_Lptr, s->lu_colp, lu, r, zp);
   }
   }
@@ -744,11 +765,11 @@ static int ilu_apply_t(Sim *s, const T *lu, const TR *r, T *zpo = nullptr) {
     if (r1 <= r0) continue;
     if (c == last && s->lu_cmaxlen[c] > kLongRow) continue;   // done with the forward launch
     if (s->lu_cmaxlen[c] > kLongRow)
-      DP_LAUNCH(s, k_ilu_bwd_w<T>, nblk(32LL * (r1 - r0)), kBlock, 0, r0, r1, nL, n,
-                s->lu_Uptr, s->lu_colp, lu, zp);
+      DP_LAUNCH_PDL(s, kPdlSmall, k_ilu_bwd_w<T>, nblk(32LL * (r1 - r0)), kBlock, 0, r0, r1, nL, n,
+                s->lu_Uptr, s->lu_colp, lu, zp, small_trig(s));
     else
-      DP_LAUNCH(s, k_ilu_bwd_r<T>, nblk((r1 - r0 + kRes - 1) / kRes), kBlock, 0, r0, r1, nL, n,
-                s->lu_Uptr, s->lu_colp, lu, zp);
+      DP_LAUNCH_PDL(s, kPdlSmall, k_ilu_bwd_r<T>, nblk((r1 - r0 + kRes - 1) / kRes), kBlock, 0, r0, r1, nL, n,
+                s->lu_Uptr, s->lu_colp, lu, zp, small_trig(s));
   }
   return DP_OK;
 }
@@ -767,7 +788,9 @@ __global__ void __launch_bounds__(kBlock) k_ilu_result(int n, const int *__restr
                                                        double *__restrict__ out,
                                                        T *__restrict__ outT,
                                                        const float *__restrict__ inj,
-                                                       int inj_perm, const T *__restrict__ zb) {
+                                                       int inj_perm, const T *__restrict__ zb, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   k_ilu_result_b<T>(blockIdx.x, gridDim.x, n, iperm, zp, base, out, outT, inj, inj_perm, zb);
 }
 
@@ -781,8 +804,8 @@ static int ilu_result(Sim *s, const double *base, double *out, T *outT = nullptr
                       const float *inj = nullptr, int inj_perm = 0, const T *zb = nullptr,
                       const T *zp = nullptr) {
   int n = s->K.n;
-  DP_LAUNCH(s, k_ilu_result<T>, nblk((n + kRes - 1) / kRes), kBlock, 0, n, s->iperm,
-            zp ? zp : reinterpret_cast<const T *>(s->ilu_zp), base, out, outT, inj, inj_perm, zb);
+  DP_LAUNCH_PDL(s, kPdlSmall, k_ilu_result<T>, nblk((n + kRes - 1) / kRes), kBlock, 0, n, s->iperm,
+            zp ? zp : reinterpret_cast<const T *>(s->ilu_zp), base, out, outT, inj, inj_perm, zb, small_trig(s));
   return DP_OK;
 }
 
@@ -793,29 +816,6 @@ int ilu_apply(Sim *s, const double *r, double *z) {
 
 // ---------------------------------------------------------------- AMG cycle
 
-
-// One colour of Gauss-Seidel: x_i = (b_i - sum_{j != i} a_ij x_j) / a_ii,
-// evaluated as x_i + (b_i - (A x)_i) / a_ii with 1/a_ii precomputed per level
-// (0 where a_ii = 0: the row is left as is).
-template <int G, typename T, typename TV = T>
-__global__ void __launch_bounds__(kBlock) k_gs_colour(int r0, int r1, const int *__restrict__ clist,
-                                                      const int *__restrict__ rowptr,
-                                                      const int *__restrict__ col,
-                                                      const TV *__restrict__ val,
-                                                      const T *__restrict__ dinv,
-                                                      const T *__restrict__ b, T *x) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  int q = r0 + t / G, lane = t % G;
-  bool valid = q < r1;
-  int i = valid ? clist[q] : 0;
-  int e0 = valid ? rowptr[i] : 0, e1 = valid ? rowptr[i + 1] : 0;
-  T s = row_dot<G, T, TV>(e0, e1, lane, col, val, x);
-  if (G > 1) s = group_sum<G, T>(s);
-  if (valid && lane == 0) {
-    T di = dinv[i];
-    if (di != T(0)) x[i] = fma(b[i] - s, di, x[i]);
-  }
-}
 
 // ---- the V-cycle's transfer and coarse-level kernels as programmatic
 // dependents (launched by DP_LAUNCH_PDL): each loads what no kernel of a
@@ -874,6 +874,45 @@ __device__ __forceinline__ T row_dot_head(const RowHead<G, T, TV> &h, const int 
     if (e + 2 * G < e1) s0 = fma(h.v[2], X(h.c[2]), s0);
   }
   return (s0 + s1) + (s2 + s3);
+}
+
+// One colour of Gauss-Seidel: x_i = (b_i - sum_{j != i} a_ij x_j) / a_ii,
+// evaluated as x_i + (b_i - (A x)_i) / a_ii with 1/a_ii precomputed per level
+// (0 where a_ii = 0: the row is left as is).  A colour of a mid-size level
+// is a few thousand rows, so the launch is a chain of dependent loads (row,
+// its bounds, entries, gathers); all but the gathers come before the wait
+// and overlap the colour before (level 1 of the 200k-cell model, 12 colours
+// over 29879 rows, 22 launches a V-cycle: 6.5 us a launch instead of 8.2).
+template <int G, typename T, typename TV = T>
+__global__ void __launch_bounds__(kBlock) k_gs_colour(int r0, int r1, const int *__restrict__ clist,
+                                                      const int *__restrict__ rowptr,
+                                                      const int *__restrict__ col,
+                                                      const TV *__restrict__ val,
+                                                      const T *__restrict__ dinv, const T *b,
+                                                      T *x, int trig) {
+  int t = blockIdx.x * blockDim.x + threadIdx.x;
+  int q = r0 + t / G, lane = t % G;
+  bool valid = q < r1;
+  int i = valid ? __ldg(clist + q) : 0;
+  int e0 = valid ? __ldg(rowptr + i) : 0, e1 = valid ? __ldg(rowptr + i + 1) : 0;
+  RowHead<G, T, TV> h;
+  h.load(e0, e1, lane, col, val);
+  T di = valid && lane == 0 ? __ldg(dinv + i) : T(0);
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
+  T s = row_dot_head<G>(h, col, val, [&](int c) { return x[c]; });
+  if (G > 1) s = group_sum<G, T>(s);
+  if (valid && lane == 0) {
+    if (di != T(0)) x[i] = fma(b[i] - s, di, x[i]);
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kBlock) k_zero(int n, T *x, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) x[i] = T(0);
 }
 
 // l1-Jacobi pre-smoothing from x = 0 fused with the residual: x_i = b_i d_i
@@ -969,7 +1008,9 @@ __global__ void __launch_bounds__(kBlock) k_csr_resid(int n, const int *__restri
                                                       const int *__restrict__ col,
                                                       const TV *__restrict__ val,
                                                       const T *__restrict__ b,
-                                                      const T *__restrict__ x, T *__restrict__ r) {
+                                                      const T *__restrict__ x, T *__restrict__ r, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   int i = t / G, lane = t % G;
   bool valid = i < n;
@@ -1033,13 +1074,13 @@ static int csr_resid(Sim *s, const Level &L, const T *b, const T *x, T *r) {
   long long thr = (long long)L.n * L.G;
   if constexpr (std::is_same<T, float>::value) {
     if (use_bf16<T>(L.valh)) {
-      DP_SWITCH_G(L.G, DP_LAUNCH(s, (k_csr_resid<GG, float, __nv_bfloat16>), nblk(thr), kBlock, 0,
-                                 L.n, L.rowptr, L.col, L.valh, b, x, r));
+      DP_SWITCH_G(L.G, DP_LAUNCH_PDL(s, kPdlSmall, (k_csr_resid<GG, float, __nv_bfloat16>), nblk(thr), kBlock, 0,
+                                 L.n, L.rowptr, L.col, L.valh, b, x, r, small_trig(s)));
       return DP_OK;
     }
   }
-  DP_SWITCH_G(L.G, DP_LAUNCH(s, (k_csr_resid<GG, T>), nblk(thr), kBlock, 0, L.n, L.rowptr, L.col,
-                             LV<T>::val(L), b, x, r));
+  DP_SWITCH_G(L.G, DP_LAUNCH_PDL(s, kPdlSmall, (k_csr_resid<GG, T>), nblk(thr), kBlock, 0, L.n, L.rowptr, L.col,
+                             LV<T>::val(L), b, x, r, small_trig(s)));
   return DP_OK;
 }
 
@@ -1201,8 +1242,11 @@ __global__ void k_dense_inverse(int n, const double *a, const int *piv, double *
 // Rows are not moved: order[i] is the step that took row i as its pivot.
 // In step k warp 0 updates column k + 1 first, picks its pivot (largest
 // magnitude, NaN never, the first free row when there is none) and forms its
-// multipliers, while the other warps update columns k + 2 on: one barrier a
-// step.  Output: lu column-major in pivot order (leading dimension ldo, even,
+// multipliers, while other warps update columns k + 2 on: one barrier a
+// step.  An FP64 instruction holds a quarter of the SM for 64 cycles, so the
+// pivot warp shares its quarter with no updating warp and divides once a
+// step (97 rows: 474 us with a division a multiplier and every warp
+// updating, 229 us so).  Output: lu column-major in pivot order (leading dimension ldo, even,
 // so that the columns can be read as 16-byte words), prow[k] the row of
 // pivot k, rdiag[k] its reciprocal (0 for a zero pivot, whose multipliers
 // are then 0 as well).
@@ -1254,7 +1298,7 @@ __global__ void __launch_bounds__(kFactorThreads) k_dense_factor(int n, const in
     __syncwarp();
     for (int i = lane; i < n; i += 32)
       if (order[i] == n) {
-        double l = d != 0.0 ? A[i * ld + k] / d : 0.0;
+        double l = A[i * ld + k] * r;
         A[i * ld + k] = l;
         mult[(k & 1) * n + i] = l;
       }
@@ -1270,8 +1314,8 @@ __global__ void __launch_bounds__(kFactorThreads) k_dense_factor(int n, const in
         if (order[i] == n) A[i * ld + k + 1] -= l[i] * uk;
       __syncwarp();
       panel(k + 1);
-    } else {
-      for (int i = warp - 1; i < n; i += kWarps - 1) {
+    } else if (warp & 3) {   // warp 0 has its quarter of the SM's FP64 units to itself
+      for (int i = warp - 1 - (warp >> 2); i < n; i += kWarps * 3 / 4) {
         if (order[i] <= k) continue;   // the pivot of step k + 1 may be marked meanwhile
         double li = l[i];
         for (int j = k + 2 + lane; j < n; j += 32) A[i * ld + j] -= li * u[j];
@@ -1626,17 +1670,25 @@ __global__ void __launch_bounds__(kBlock) k_gs_c(int r0, int r1, const int *__re
                                                  const int *__restrict__ colp,
                                                  const T *__restrict__ pv,
                                                  const T *__restrict__ dinv,
-                                                 const T *__restrict__ b, T *x) {
+                                                 const T *__restrict__ b, T *x, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   k_gs_c_b<T>(blockIdx.x, gridDim.x, r0, r1, rowptr, colp, pv, dinv, b, x);
 }
 
-// The first colour of a Gauss-Seidel sweep that starts from x = 0: every
-// x_j a row reads is still zero, so the row formula reduces to
-// x_i = fma(b_i, 1/a_ii, 0) (the same value bit for bit: the sum is +0).
+// The start of a Gauss-Seidel sweep from x = 0: on the first colour's rows
+// [r0, r1) every x_j a row reads is still zero, so the row formula reduces
+// to x_i = fma(b_i, 1/a_ii, 0) (the same value bit for bit: the sum is +0);
+// the other rows' x = 0.
 template <typename T>
-__global__ void k_gs_c_first(int r0, int r1, const T *__restrict__ dinv, const T *__restrict__ b,
-                             T *__restrict__ x) {
-  k_gs_c_first_b<T>(blockIdx.x, gridDim.x, r0, r1, dinv, b, x);
+__global__ void __launch_bounds__(kBlock) k_gs_c_start(int n, int r0, int r1, const T *__restrict__ dinv,
+                                                       const T *b, T *__restrict__ x, int trig) {
+  int q = blockIdx.x * blockDim.x + threadIdx.x;
+  bool in = q >= r0 && q < r1;
+  T di = in ? __ldg(dinv + q) : T(0);
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
+  if (q < n) x[q] = di != T(0) ? fma(b[q] - T(0), di, T(0)) : T(0);
 }
 
 
@@ -1704,7 +1756,9 @@ __global__ void __launch_bounds__(kBlock) k_resid_c(int r0, int r1, const int *_
                                                     const int *__restrict__ colp,
                                                     const T *__restrict__ pv,
                                                     const T *__restrict__ b,
-                                                    const T *__restrict__ x, T *__restrict__ r) {
+                                                    const T *__restrict__ x, T *__restrict__ r, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   k_resid_c_b<T>(blockIdx.x, gridDim.x, r0, r1, rowptr, colp, pv, b, x, r);
 }
 
@@ -1981,7 +2035,7 @@ static void sweep_tma(Sim *s, int G, int r0, int r1, const T *pv, const T *dinv,
 // warp walks all of the sweep's tiles without waiting at the barriers (the
 // matrix does not change), so the next colour's tiles are already in
 // shared memory when its phase starts.  Long-row colours (the wells) take a
-// consumer warp per row.  Every row's arithmetic is that of k_gs_c_first,
+// consumer warp per row.  Every row's arithmetic is that of k_gs_c_start,
 // k_gs_c and k_gs_c_wp, so the sweep's result is theirs bit for bit.  The
 // barrier counts arrivals on bar[0] (the k-th barrier is passed at (k+1)
 // gridDim.x arrivals) and the last CTA to finish resets it (with bar[1],
@@ -2188,7 +2242,7 @@ static int l0_lanes(const Sim *s) {
 }
 
 // from_zero: x = 0 on entry (the pre-smoothing), so the first colour is the
-// reduced formula of k_gs_c_first; preset: the kernel that wrote b has also
+// reduced formula of k_gs_c_start; preset: the kernel that wrote b has also
 // written that x (X0Init), so the sweep starts with the second colour
 template <typename T>
 static int gs_sweep_c(Sim *s, const T *b, T *x, bool forward, bool from_zero = false,
@@ -2222,8 +2276,6 @@ static int gs_sweep_c(Sim *s, const T *b, T *x, bool forward, bool from_zero = f
     return gs_sweep_persistent<T, 3, 6>(s, plan, L0C<T>::pv(s), L0C<T>::dinv(s), b, x);
   }
   if (G <= -4) G = 1;
-  if (from_zero && !preset)
-    DP_CUDA(s, cudaMemsetAsync(x, 0, (size_t)s->lu_cstart[nc] * sizeof(T), s->stream));
   std::vector<int> order;   // the non-empty colours in sweep order
   for (int t = 0; t < nc; ++t) {
     int c = forward ? t : nc - 1 - t;
@@ -2237,7 +2289,8 @@ static int gs_sweep_c(Sim *s, const T *b, T *x, bool forward, bool from_zero = f
     if (first) {
       first = false;
       if (!preset)
-        DP_LAUNCH(s, k_gs_c_first<T>, nblk(r1 - r0), kBlock, 0, r0, r1, L0C<T>::dinv(s), b, x);
+        DP_LAUNCH_PDL(s, kPdlSmall, k_gs_c_start<T>, nblk(s->lu_cstart[nc]), kBlock, 0,
+                      s->lu_cstart[nc], r0, r1, L0C<T>::dinv(s), b, x, small_trig(s));
       continue;
     }
     if (lng(c))
@@ -2253,8 +2306,8 @@ static int gs_sweep_c(Sim *s, const T *b, T *x, bool forward, bool from_zero = f
     else if (G < 0)
       sweep_tma<T>(s, G, r0, r1, L0C<T>::pv(s), L0C<T>::dinv(s), b, x, nullptr);
     else
-      DP_LAUNCH(s, k_gs_c<T>, nblk(r1 - r0), kBlock, 0, r0, r1, s->lu_rowptr, s->l0_colp,
-                L0C<T>::pv(s), L0C<T>::dinv(s), b, x);
+      DP_LAUNCH_PDL(s, kPdlSmall, k_gs_c<T>, nblk(r1 - r0), kBlock, 0, r0, r1, s->lu_rowptr, s->l0_colp,
+                L0C<T>::pv(s), L0C<T>::dinv(s), b, x, small_trig(s));
   }
   return DP_OK;
 }
@@ -2283,8 +2336,8 @@ static int resid_c(Sim *s, const T *b, const T *x, T *r) {
       else if (G < 0)
         sweep_tma<T>(s, G, r0, r1, L0C<T>::pv(s), nullptr, b, (T *)x, r);
       else
-        DP_LAUNCH(s, k_resid_c<T>, nblk(r1 - r0), kBlock, 0, r0, r1, s->lu_rowptr, s->l0_colp,
-                  L0C<T>::pv(s), b, x, r);
+        DP_LAUNCH_PDL(s, kPdlSmall, k_resid_c<T>, nblk(r1 - r0), kBlock, 0, r0, r1, s->lu_rowptr, s->l0_colp,
+                  L0C<T>::pv(s), b, x, r, small_trig(s));
     }
     c = c1;
   }
@@ -2319,14 +2372,16 @@ static int gs_sweep(Sim *s, Level &L, const T *b, T *x, bool forward) {
       bool done = false;
       if constexpr (std::is_same<T, float>::value) {
         if (use_bf16<T>(L.valh)) {
-          DP_SWITCH_G(L.G, DP_LAUNCH(s, (k_gs_colour<GG, float, __nv_bfloat16>), nblk(thr), kBlock,
-                                     0, r0, r1, L.clist, L.rowptr, L.col, L.valh, L.dinvf, b, x));
+          DP_SWITCH_G(L.G, DP_LAUNCH_PDL(s, kPdlSmall, (k_gs_colour<GG, float, __nv_bfloat16>),
+                                         nblk(thr), kBlock, 0, r0, r1, L.clist, L.rowptr, L.col,
+                                         L.valh, L.dinvf, b, x, small_trig(s)));
           done = true;
         }
       }
       if (!done)
-        DP_SWITCH_G(L.G, DP_LAUNCH(s, (k_gs_colour<GG, T>), nblk(thr), kBlock, 0, r0, r1, L.clist,
-                                   L.rowptr, L.col, LV<T>::val(L), LV<T>::dinv(L), b, x));
+        DP_SWITCH_G(L.G, DP_LAUNCH_PDL(s, kPdlSmall, (k_gs_colour<GG, T>), nblk(thr), kBlock, 0,
+                                       r0, r1, L.clist, L.rowptr, L.col, LV<T>::val(L),
+                                       LV<T>::dinv(L), b, x, small_trig(s)));
     }
   }
   return DP_OK;
@@ -2376,7 +2431,7 @@ static int vcycle_r(Sim *s, int l, const T *b, T *x, const T **res, bool x_prese
       *res = LV<T>::r(L);
       return DP_OK;
     }
-    DP_CUDA(s, cudaMemsetAsync(x, 0, (size_t)n * sizeof(T), s->stream));
+    DP_LAUNCH_PDL(s, kPdlSmall, k_zero<T>, nblk(n), kBlock, 0, n, x, small_trig(s));
     DP_TRY(gs_sweep<T>(s, L, b, x, true));
     DP_TRY(gs_sweep<T>(s, L, b, x, false));
     return DP_OK;
@@ -2386,7 +2441,7 @@ static int vcycle_r(Sim *s, int l, const T *b, T *x, const T **res, bool x_prese
   if (L.l1) {
     DP_TRY(jacobi_pre<T>(s, L, b, x, r));
   } else {
-    DP_CUDA(s, cudaMemsetAsync(x, 0, (size_t)n * sizeof(T), s->stream));
+    DP_LAUNCH_PDL(s, kPdlSmall, k_zero<T>, nblk(n), kBlock, 0, n, x, small_trig(s));
     DP_TRY(gs_sweep<T>(s, L, b, x, true));
     DP_TRY(csr_resid<T>(s, L, b, x, r));
   }
@@ -2475,8 +2530,8 @@ static int tune_level(Sim *s, int l, int reps, std::string &rep) {
                                    0, L.n, L.rowptr, L.col, LV<T>::val(L), LV<T>::dinv(L), b, x,
                                    r, (int)pdl_trigger()));
     } else {
-      DP_SWITCH_G(g, DP_LAUNCH(s, (k_csr_resid<GG, T>), nblk(thr), kBlock, 0, L.n, L.rowptr,
-                               L.col, LV<T>::val(L), b, x, r));
+      DP_SWITCH_G(g, DP_LAUNCH_PDL(s, kPdlSmall, (k_csr_resid<GG, T>), nblk(thr), kBlock, 0, L.n, L.rowptr,
+                               L.col, LV<T>::val(L), b, x, r, small_trig(s)));
     }
     return DP_OK;
   };
@@ -2586,7 +2641,9 @@ int autotune(Sim *s, int reps, std::string &rep) {
 // z1 = F r;  z2 = z1 + P V(R (r - A z1));  z = z2 + F (r - A z2)
 
 template <typename T>
-__global__ void k_inject_add(int n, const T *xp, double *z, const int *imap) {
+__global__ void k_inject_add(int n, const T *xp, double *z, const int *imap, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) z[2 * i] += double(xp[imap ? __ldg(imap + i) : i]);
 }
@@ -2594,7 +2651,9 @@ __global__ void k_inject_add(int n, const T *xp, double *z, const int *imap) {
 // The injection into the FP32 copy of z1 only (updated in FP32: no
 // conversions on the FP64 pipe); the FP64 z1 takes the same correction in
 // the final result gather (ilu_result's inj).
-__global__ void k_inject_f32(int n, const float *xp, float *zf, const int *imap) {
+__global__ void k_inject_f32(int n, const float *xp, float *zf, const int *imap, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   k_inject_f32_b(blockIdx.x, gridDim.x, n, xp, zf, imap);
 }
 
@@ -2603,7 +2662,9 @@ __global__ void k_inject_f32(int n, const float *xp, float *zf, const int *imap)
 // in that order), the other is z1's; the same sum as k_inject_f32's.
 __global__ void __launch_bounds__(kBlock) k_inject_colour_f32(int n, const float2 *__restrict__ z1,
                                                               const float *__restrict__ xp,
-                                                              float2 *__restrict__ z2) {
+                                                              float2 *__restrict__ z2, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= n) return;
   float2 v = z1[q];
@@ -2630,10 +2691,10 @@ int cpr_apply(Sim *s, const double *r, double *z) {
     if (s->opt.precond == 1) return ilu_apply(s, r, z);
     DP_TRY(ilu_apply(s, r, s->z1));
     const int *m = l0c_on(s) ? s->iperm : nullptr;   // level-0 vectors in colour order
-    DP_LAUNCH(s, k_bsr_presid, 1 + nblk(s->sv_long0), kBlock, 0, nb, s->sv_sL, s->sv_sc,
-              s->sv_long0, s->srowptr, s->scol, s->sa00, s->sa01, s->z1, r, s->rp, m);
+    DP_LAUNCH_PDL(s, kPdlSmall, k_bsr_presid, 1 + nblk(s->sv_long0), kBlock, 0, nb, s->sv_sL, s->sv_sc,
+              s->sv_long0, s->srowptr, s->scol, s->sa00, s->sa01, s->z1, r, s->rp, m, small_trig(s));
     DP_TRY(vcycle(s, 0, s->rp, s->xp));
-    DP_LAUNCH(s, k_inject_add<double>, nblk(nb), kBlock, 0, nb, s->xp, s->z1, m);
+    DP_LAUNCH_PDL(s, kPdlSmall, k_inject_add<double>, nblk(nb), kBlock, 0, nb, s->xp, s->z1, m, small_trig(s));
     DP_TRY(bsr_residual(s, r, s->z1, s->r1));
     DP_TRY((ilu_apply_t<double, double>(s, s->lu_val, s->r1)));
     return ilu_result<double>(s, s->z1, z);           // z = z2 + F (r - A z2)
@@ -2670,20 +2731,20 @@ int cpr_apply(Sim *s, const double *r, double *z) {
       xi.f1 = s->lu_cstart[f + 1];
     }
   }
-  DP_LAUNCH(s, k_bsr_presid_f32, 1 + nblk(s->sv_long0), kBlock, 0, nb, s->sv_sL, s->sv_sc,
+  DP_LAUNCH_PDL(s, kPdlSmall, k_bsr_presid_f32, 1 + nblk(s->sv_long0), kBlock, 0, nb, s->sv_sL, s->sv_sc,
             s->sv_long0, s->srowptr, scs, reinterpret_cast<const float2 *>(s->spf), z1s, r, L0.bf,
-            m, xi);
+            m, xi, small_trig(s));
   DP_TRY(vcycle_t<float>(s, 0, L0.bf, L0.xf, xi.x != nullptr));
   const float *z2s = s->z1f;
   if (cz) {
-    DP_LAUNCH(s, k_inject_colour_f32, nblk(nb), kBlock, 0, nb,
-              reinterpret_cast<const float2 *>(s->ilu_zp), L0.xf, reinterpret_cast<float2 *>(s->z2c));
+    DP_LAUNCH_PDL(s, kPdlSmall, k_inject_colour_f32, nblk(nb), kBlock, 0, nb,
+              reinterpret_cast<const float2 *>(s->ilu_zp), L0.xf, reinterpret_cast<float2 *>(s->z2c), small_trig(s));
     z2s = s->z2c;
   } else {
-    DP_LAUNCH(s, k_inject_f32, nblk(nb), kBlock, 0, nb, L0.xf, s->z1f, m);
+    DP_LAUNCH_PDL(s, kPdlSmall, k_inject_f32, nblk(nb), kBlock, 0, nb, L0.xf, s->z1f, m, small_trig(s));
   }
-  DP_LAUNCH(s, k_bsr_resid_f32, 1 + nblk(2LL * s->sv_long0), kBlock, 0, nb, s->sv_sL, s->sv_sc,
-            s->sv_long0, s->srowptr, scs, s->svalf, z2s, r, s->r1f);
+  DP_LAUNCH_PDL(s, kPdlSmall, k_bsr_resid_f32, 1 + nblk(2LL * s->sv_long0), kBlock, 0, nb, s->sv_sL, s->sv_sc,
+            s->sv_long0, s->srowptr, scs, s->svalf, z2s, r, s->r1f, small_trig(s));
   float *zp2 = reinterpret_cast<float *>(s->ilu_zp2);
   DP_TRY((ilu_apply_t<float, float>(s, s->lu_valf, s->r1f, zp2)));
   // z = z2 + F (r - A z2), z2 = z1 + P e formed here (z1 from the first result)
@@ -2704,7 +2765,9 @@ __global__ void __launch_bounds__(kBlock, kDotBlocks / 152) k_multidot(long long
                                                      long long ldv,
                                                      const double *__restrict__ w,
                                                      double *__restrict__ part, int part_off,
-                                                     const double *__restrict__ gate) {
+                                                     const double *__restrict__ gate, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   k_multidot_b<NV, SELF>(blockIdx.x, gridDim.x, N, V, ldv, w, part, part_off, gate);
 }
 
@@ -2721,7 +2784,9 @@ __global__ void __launch_bounds__(kBlock, kDotBlocks / 152) k_multidot(long long
 // the eight group sums are then added in group order.
 __global__ void __launch_bounds__(256) k_dot_final(const double *part, int nblocks, int nv,
                                                    double *dots, double *H, int m, int j,
-                                                   int mode, double *scal, double reorth) {
+                                                   int mode, double *scal, double reorth, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   k_dot_final_b(blockIdx.x, gridDim.x, part, nblocks, nv, dots, H, m, j, mode, scal, reorth);
 }
 
@@ -2734,7 +2799,9 @@ __global__ void __launch_bounds__(kBlock) k_project(long long N, const double *_
                                                     const double *__restrict__ c,
                                                     double *__restrict__ w,
                                                     double *__restrict__ out,
-                                                    const double *__restrict__ scal, int pass) {
+                                                    const double *__restrict__ scal, int pass, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   k_project_b(blockIdx.x, gridDim.x, N, V, ldv, nv, c, w, out, scal, pass);
 }
 
@@ -2755,7 +2822,9 @@ __global__ void k_scale(long long N, const double *x, const double *alpha, int i
 // Givens rotations on column j of the Hessenberg matrix and the rotated
 // right-hand side g; res_out = |g_{j+1}|.
 __global__ void k_givens(double *H, double *cs, double *sn, double *g, int m, int j,
-                         double *res_out) {
+                         double *res_out, int trig) {
+  griddep_wait();
+  if (trig) griddep_launch_dependents();
   k_givens_b(blockIdx.x, gridDim.x, H, cs, sn, g, m, j, res_out);
 }
 
@@ -2779,19 +2848,19 @@ static int dots(Sim *s, const double *V, long long ldv, int nv, const double *w,
 #define DP_MD(NVC)                                                                             \
   case NVC:                                                                                    \
     if (mode >= 3 && v0 == 0)                                                                  \
-      DP_LAUNCH(s, (k_multidot<NVC, true>), nblocks, kBlock, 0, N, Vb, ldv, w, s->dots_part,   \
-                v0, gate);                                                                     \
+      DP_LAUNCH_PDL(s, kPdlSmall, (k_multidot<NVC, true>), nblocks, kBlock, 0, N, Vb, ldv, w, s->dots_part,   \
+                v0, gate, small_trig(s));                                                                     \
     else                                                                                       \
-      DP_LAUNCH(s, (k_multidot<NVC, false>), nblocks, kBlock, 0, N, Vb, ldv, w,                \
-                s->dots_part, v0, gate);                                                       \
+      DP_LAUNCH_PDL(s, kPdlSmall, (k_multidot<NVC, false>), nblocks, kBlock, 0, N, Vb, ldv, w,                \
+                s->dots_part, v0, gate, small_trig(s));                                                       \
     break;
     switch (cnt) {
       DP_MD(1) DP_MD(2) DP_MD(3) DP_MD(4) DP_MD(5) DP_MD(6) DP_MD(7) DP_MD(8)
     }
 #undef DP_MD
   }
-  DP_LAUNCH(s, k_dot_final, 1, 256, 0, s->dots_part, nblocks, nv, s->dots, s->H, s->m, j, mode,
-            s->scal, s->opt.reorth);
+  DP_LAUNCH_PDL(s, kPdlSmall, k_dot_final, 1, 256, 0, s->dots_part, nblocks, nv, s->dots, s->H, s->m, j, mode,
+            s->scal, s->opt.reorth, small_trig(s));
   return DP_OK;
 }
 
@@ -2799,10 +2868,10 @@ static int dots(Sim *s, const double *V, long long ldv, int nv, const double *w,
 static int norm_into(Sim *s, const double *x, double *dst) {
   long long N = 2LL * s->K.n;
   int nblocks = dot_blocks(N);
-  DP_LAUNCH(s, (k_multidot<1, false>), nblocks, kBlock, 0, N, x, 0LL, x, s->dots_part, 0,
-            (const double *)nullptr);
-  DP_LAUNCH(s, k_dot_final, 1, 256, 0, s->dots_part, nblocks, 1, dst, s->H, s->m, 0, 0, s->scal,
-            0.0);
+  DP_LAUNCH_PDL(s, kPdlSmall, (k_multidot<1, false>), nblocks, kBlock, 0, N, x, 0LL, x, s->dots_part, 0,
+            (const double *)nullptr, small_trig(s));
+  DP_LAUNCH_PDL(s, kPdlSmall, k_dot_final, 1, 256, 0, s->dots_part, nblocks, 1, dst, s->H, s->m, 0, 0, s->scal,
+            0.0, small_trig(s));
   return DP_OK;
 }
 
@@ -2825,10 +2894,10 @@ static int arnoldi_step(Sim *s, int j) {
   DP_TRY(cpr_apply(s, vj, zj));
   DP_TRY(bsr_spmv(s, zj, s->w));
   DP_TRY(dots(s, s->V, N, j + 1, s->w, 3, j));
-  DP_LAUNCH(s, k_project, gridN, kBlock, 0, N, s->V, N, j + 1, s->dots, s->w, vnext, s->scal, 0);
+  DP_LAUNCH_PDL(s, kPdlSmall, k_project, gridN, kBlock, 0, N, s->V, N, j + 1, s->dots, s->w, vnext, s->scal, 0, small_trig(s));
   DP_TRY(dots(s, s->V, N, j + 1, s->w, 4, j, s->scal + 4));
-  DP_LAUNCH(s, k_project, gridN, kBlock, 0, N, s->V, N, j + 1, s->dots, s->w, vnext, s->scal, 1);
-  DP_LAUNCH(s, k_givens, 1, 32, 0, s->H, s->cs, s->sn, s->g, m, j, s->scal + 3);
+  DP_LAUNCH_PDL(s, kPdlSmall, k_project, gridN, kBlock, 0, N, s->V, N, j + 1, s->dots, s->w, vnext, s->scal, 1, small_trig(s));
+  DP_LAUNCH_PDL(s, kPdlSmall, k_givens, 1, 32, 0, s->H, s->cs, s->sn, s->g, m, j, s->scal + 3, small_trig(s));
   return DP_OK;
 }
 
@@ -2937,6 +3006,7 @@ int fgmres(Sim *s, double tol, int *iters, double *relres) {
 int la_alloc(Sim *s) {
   int m = std::max(1, std::min(s->opt.gmres_restart, 30));
   s->m = m;
+  s->pdl_small = s->K.n <= kPdlSmallRows;
   long long N = 2LL * s->K.n;
   s->V = (double *)dalloc(s, (size_t)(m + 1) * N * 8);
   s->Z = (double *)dalloc(s, (size_t)m * N * 8);

@@ -61,3 +61,28 @@ def test_cluster_cycle_from_level_0(coarse_max):
     prob = di.tiny()
     g, o = relres(prob, 3, interior(prob, 5), amg_coarse_max=coarse_max)
     assert abs(g - o) <= 1e-6 * o + 1e-12
+
+
+def test_small_realisations_dependent_launches_change_no_result():
+    """Every kernel of an Arnoldi step as a programmatic dependent (DPSIM_PDL
+    63, the default) or that class off (31): the same state, bit for bit, in a
+    child process each."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    code = ("import sys; sys.path.insert(0, sys.argv[1])\n"
+            "import dp_inputs as di, numpy as np\n"
+            "from paper_1808_04338_gb300 import dpsim\n"
+            "h = []\n"
+            "for prob, mode, kw in ((di.tiny(), 'parity', {}), (di.layered(31, 29, 6), 'parity', {}),\n"
+            "                       (di.layered(47, 45, 5), 'report', dict(precision=1)),\n"
+            "                       (di.layered(47, 45, 5), 'report', dict(precision=2, schur=1))):\n"
+            "    s = dpsim.Sim(prob, dpsim.options(mode, **kw))\n"
+            "    rc, st = s.advance(prob.dt)\n"
+            "    assert rc == 0\n"
+            "    h += [a.tobytes().hex() for a in s.get_state()] + [st.linear_iters]\n"
+            "import hashlib; print(hashlib.sha256(repr(h).encode()).hexdigest())\n")
+    out = [subprocess.run([sys.executable, "-c", code, root], capture_output=True, text=True,
+                          env=dict(os.environ, DPSIM_PDL=m), check=True).stdout for m in ("63", "31")]
+    assert out[0] == out[1] and len(out[0].strip()) == 64
