@@ -311,9 +311,11 @@ struct Sim {
   double *p = nullptr, *sw = nullptr, *bhp = nullptr;
   double *pn = nullptr, *swn = nullptr, *bhpn = nullptr, *Mn = nullptr;
   double *R = nullptr, *bh = nullptr, *y = nullptr;
-  double *pr = nullptr;                              // cell properties, 8 x nc (SoA)
-  double *fconn = nullptr;   // per connection (3 faces a location, then its f-m link): F
-  int *atpos = nullptr;      // position of the transposed block of each Jacobian entry
+  double *pr = nullptr;      // cell properties, 8 or (with capillary curves) 10 arrays of nc
+  // per connection (faces along x, y, z, then the f-m links, nL each): the
+  // fluxes F, the positions of its two blocks, its transmissibility
+  double *fconn = nullptr, *ctrans = nullptr;
+  int2 *cpos = nullptr;
   double *Macc = nullptr;                            // phase masses at the iterate, 2 x nc
   double dt = 1.0, inv_dt = 1.0;
   double *norm_part = nullptr;                       // reduction partials

@@ -304,7 +304,7 @@ extern "C" int sim_create(const dp_grid *grid, const dp_rock *rock, const dp_flu
   s->Mn = (double *)dalloc(s, 2 * nc8);
   s->R = (double *)dalloc(s, nb16); s->bh = (double *)dalloc(s, nb16);
   s->y = (double *)dalloc(s, nb16);
-  s->pr = (double *)dalloc(s, 8 * nc8);
+  s->pr = (double *)dalloc(s, (P.pc_n[0] > 0 || P.pc_n[1] > 0 ? 10 : 8) * nc8);
   s->Macc = (double *)dalloc(s, 2 * nc8);
   s->norm_blocks = std::min(nblk(P.nb), 1024);
   s->norm_part = (double *)dalloc(s, (size_t)s->norm_blocks * 64);

@@ -86,3 +86,35 @@ def test_small_realisations_dependent_launches_change_no_result():
     out = [subprocess.run([sys.executable, "-c", code, root], capture_output=True, text=True,
                           env=dict(os.environ, DPSIM_PDL=m), check=True).stdout for m in ("63", "31")]
     assert out[0] == out[1] and len(out[0].strip()) == 64
+
+
+@pytest.mark.parametrize("gravity", [0.0, 9.80665])
+@pytest.mark.parametrize("capillary", [False, True])
+@pytest.mark.parametrize("swc_fraction", [0.0, 0.5, 1.0])
+def test_assembly_with_resting_phases_bit_exact(gravity, capillary, swc_fraction):
+    """J and R bit for bit, signs of zeros included, where a phase is at its
+    residual saturation (its flux terms are left out) in none, half or all of
+    the cells, for both flow directions; three kinds of wells, one of them
+    with more perforations than a warp has lanes."""
+    from test_gpu_parity import with_pc
+    prob = small(6, 5, 40, wells="none", g=gravity)
+    prob.wells = [di.Well(di.WELL_RATE_INJ, 0, 0, 0, 39, 100.0 * di.BBL_DAY),
+                  di.Well(di.WELL_BHP, 5, 4, 3, 3, 2500.0 * di.PSI),
+                  di.Well(di.WELL_OIL_RATE, 2, 2, 1, 38, 1.0, limit=15.0 * di.PSI)]
+    prob.bhp0 = np.array([3100.0, 2500.0, 2700.0]) * di.PSI
+    if capillary:
+        with_pc(prob)
+    rng = np.random.default_rng(11)
+    nc = prob.n_cells
+    p = prob.p0 + rng.uniform(-3e5, 3e5, nc)
+    p[::7] = prob.p0[::7]                      # equal pressures too
+    sw = rng.uniform(0.25, 0.75, nc)
+    rest = rng.random(nc) < swc_fraction
+    sw[rest] = np.where(rng.random(rest.sum()) < 0.5, prob.swc, 1.0 - prob.sor)
+    out = []
+    for s in (gpu().Sim(prob, gpu().options("parity")), O.OracleSim(prob, O.options("parity"))):
+        s.set_iterate(p, sw, prob.bhp0)
+        s.assemble(prob.dt)
+        out.append(s.jacobian())
+    for g, o in zip(out[0][2:], out[1][2:]):
+        assert np.array_equal(g.view(np.uint64), o.view(np.uint64))
