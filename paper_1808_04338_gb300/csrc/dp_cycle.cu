@@ -211,7 +211,9 @@ __device__ __forceinline__ float2 ld2(const float *p) {
   return __ldg(reinterpret_cast<const float2 *>(p));
 }
 // v == 0 without the FP64 pipe's comparison
-__device__ __forceinline__ bool is_zero(double v) { return (__double_as_longlong(v) << 1) == 0; }
+__device__ __forceinline__ bool is_zero(double v) {
+  return (((unsigned)__double2hiint(v) << 1) | (unsigned)__double2loint(v)) == 0u;
+}
 __device__ __forceinline__ bool is_zero(float v) { return v == 0.f; }
 
 // One Gauss-Seidel sweep over the colours of a level from its padded copy: a

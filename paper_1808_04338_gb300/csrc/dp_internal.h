@@ -48,6 +48,7 @@ struct Phys {
   double inv_span, inv_mu_o, inv_mu_w;
   double sigma, c_rock, p_ref_rock;
   double drho_o, drho_w;          // rho_ref c per phase (the density slopes)
+  int rock;                       // c_rock is not zero
   int pc_n[2];                    // capillary tables: points per continuum
   const double *pc_tab[2];        //   device (s_w, p_cow) pairs, or null
 };

@@ -9,6 +9,7 @@
 // processor that evaluated them.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "dp_internal.h"
 
@@ -16,12 +17,20 @@ namespace dp {
 
 // ---------------------------------------------------------------- physics
 
-// Sign and zero tests and sign changes of doubles as integer operations: on
-// this GPU an FP64 comparison or addition costs a quarter of an SM 64 cycles.
-__device__ __forceinline__ long long bits(double v) { return __double_as_longlong(v); }
-__device__ __forceinline__ bool nonneg(double v) { return bits(v) >= 0 || (bits(v) << 1) == 0; }
+// Sign and zero tests and sign changes of doubles on their two 32-bit halves:
+// on this GPU an FP64 comparison or negation costs a quarter of an SM 64
+// cycles, and 64-bit integer forms of them are compiled back into one.
+__device__ __forceinline__ bool is_zero(double v) {
+  return (((unsigned)__double2hiint(v) << 1) | (unsigned)__double2loint(v)) == 0u;
+}
+__device__ __forceinline__ bool nonneg(double v) { return __double2hiint(v) >= 0 || is_zero(v); }
 __device__ __forceinline__ double flip(double v) {   // -v
-  return __longlong_as_double(bits(v) ^ (long long)0x8000000000000000ull);
+  return __hiloint2double(__double2hiint(v) ^ (int)0x80000000, __double2loint(v));
+}
+__device__ __forceinline__ double twice(double v) {   // 2 v, v finite and >= 0
+  int h = __double2hiint(v);
+  return h >= 0x00100000 && h < 0x7fd00000 ? __hiloint2double(h + 0x00100000, __double2loint(v))
+                                           : 2.0 * v;
 }
 
 // Cell properties (Section 2): linear densities, porosity, Corey relative
@@ -57,20 +66,26 @@ __device__ __forceinline__ void props(const Phys &P, const double *phi_f, const 
   q.drho[0] = P.rho_o_ref * P.c_o;
   q.drho[1] = P.rho_w_ref * P.c_w;
   // with no rock compressibility the factor is 1 exactly
-  q.phi = P.c_rock == 0.0 ? phi_ref : phi_ref * (1.0 + P.c_rock * (p - P.p_ref_rock));
-  q.dphi = P.c_rock == 0.0 ? 0.0 : phi_ref * P.c_rock;
+  q.phi = !P.rock ? phi_ref : phi_ref * (1.0 + P.c_rock * (p - P.p_ref_rock));
+  q.dphi = !P.rock ? 0.0 : phi_ref * P.c_rock;
   double S = (sw - P.swc) * P.inv_span, dS;
-  // S <= 0, S >= 1 (not a NaN) by their bits
-  constexpr long long kOne = 0x3ff0000000000000ll, kInf = 0x7ff0000000000000ll;
-  long long sb = bits(S);
-  if (sb == 0 || (sb < 0 && (sb & 0x7fffffffffffffffll) <= kInf)) { S = 0.0; dS = 0.0; }
-  else if (sb >= kOne && sb <= kInf) { S = 1.0; dS = 0.0; }
+  const int hi = __double2hiint(S), mag = hi & 0x7fffffff;
+  const bool nan = mag > 0x7ff00000 || (mag == 0x7ff00000 && __double2loint(S) != 0);
+  if (!nan && (hi < 0 || is_zero(S))) { S = 0.0; dS = 0.0; }        // S <= 0
+  else if (!nan && hi >= 0x3ff00000) { S = 1.0; dS = 0.0; }          // S >= 1
   else dS = P.inv_span;
+  if (is_zero(S)) {   // no mobile water: the values below, without their arithmetic
+    q.lam[1] = 0.0;
+    q.dlam[1] = 0.0;
+    q.lam[0] = P.inv_mu_o;
+    q.dlam[0] = -0.0;
+    return;
+  }
   double so = 1.0 - S;
   q.lam[1] = (S * S) * P.inv_mu_w;
-  q.dlam[1] = ((2.0 * S) * dS) * P.inv_mu_w;
+  q.dlam[1] = (twice(S) * dS) * P.inv_mu_w;
   q.lam[0] = (so * so) * P.inv_mu_o;
-  q.dlam[0] = (-((2.0 * so) * dS)) * P.inv_mu_o;
+  q.dlam[0] = flip(twice(so) * dS) * P.inv_mu_o;
 }
 
 // Phase masses V phi rho s of a cell and their derivatives [phase][p, sw].
@@ -80,14 +95,14 @@ __device__ __forceinline__ void accumulation(const Phys &P, double sw, const Pro
   double so = 1.0 - sw;
   M[0] = (Vphi * q.rho[0]) * so;
   M[1] = (Vphi * q.rho[1]) * sw;
-  if (P.c_rock == 0.0) {   // dphi = 0: the first products are exact zeros
+  if (!P.rock) {   // dphi = 0: the first products are exact zeros
     dM[0] = (P.V * (q.phi * q.drho[0])) * so;
     dM[2] = (P.V * (q.phi * q.drho[1])) * sw;
   } else {
     dM[0] = (P.V * ((q.dphi * q.rho[0]) + (q.phi * q.drho[0]))) * so;
     dM[2] = (P.V * ((q.dphi * q.rho[1]) + (q.phi * q.drho[1]))) * sw;
   }
-  dM[1] = -(Vphi * q.rho[0]);
+  dM[1] = flip(Vphi * q.rho[0]);
   dM[3] = Vphi * q.rho[1];
 }
 
@@ -408,9 +423,9 @@ int phys_build_pattern(Sim *s) {
 // few FP64 instructions; the products and sums are those of the row-by-row
 // formulas, in their order, and what is left out is exact: terms that are
 // zero because a cell is downstream, or because no water moves there.
-// 200x200x50 locations (8M unknowns): 1.28 ms for the four kernels of
-// sim_assemble's residual, Jacobian and norms instead of 1.53; 61x43x27 with
-// gravity and curves: 92 us instead of 144.
+// sim_assemble's residual, Jacobian and norms: 1.17 ms at 200x200x50
+// locations (8M unknowns) instead of 1.57, 82 us at 61x43x27 with gravity
+// and curves instead of 144.
 //
 // Cell properties stored structure-of-arrays, fracture cells then matrix
 // cells (cell c at (c & 1) nL + c / 2, so that a warp of connections along
@@ -433,12 +448,18 @@ __global__ void __launch_bounds__(kBlock) k_props(Phys P, const double *phi_f, c
   props(P, phi_f, phi_m, c, p[c], s, q);
   size_t n = (size_t)P.nc;
   double *o = pr + prop_at(P, c);
-#pragma unroll
-  for (int al = 0; al < 2; ++al) {
-    o[(3 * al) * n] = q.rho[al] * q.lam[al];
-    o[(3 * al + 1) * n] = q.drho[al] * q.lam[al];
-    o[(3 * al + 2) * n] = q.rho[al] * q.dlam[al];
-    o[(6 + al) * n] = q.rho[al];
+  o[6 * n] = q.rho[0];
+  o[7 * n] = q.rho[1];
+  o[0] = q.rho[0] * q.lam[0];
+  o[n] = q.drho[0] * q.lam[0];
+  if (is_zero(q.lam[1]) && is_zero(q.dlam[1]) && is_zero(q.dlam[0])) {
+    o[2 * n] = -0.0;   // no mobile water, densities positive
+    o[3 * n] = o[4 * n] = o[5 * n] = 0.0;
+  } else {
+    o[2 * n] = q.rho[0] * q.dlam[0];
+    o[3 * n] = q.rho[1] * q.lam[1];
+    o[4 * n] = q.drho[1] * q.lam[1];
+    o[5 * n] = q.rho[1] * q.dlam[1];
   }
   if (CAP) {
     double pc, dpc;
@@ -459,7 +480,31 @@ struct AsmArgs {
   double *val, *R, *Macc;
   double2 *fconn;
   double inv_dt;
+  bool wide;   // val on a 32-byte boundary
 };
+
+// A 2x2 block as one 32-byte access, where the blocks start on 32-byte
+// boundaries (wide; an allocator given by the caller may give less).
+__device__ __forceinline__ void store_block(double *p, const double (&v)[4], bool wide) {
+  if (wide) {
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]),
+                 "d"(v[2]), "d"(v[3])
+                 : "memory");
+  } else {
+    reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
+    reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
+  }
+}
+__device__ __forceinline__ void load_block(const double *p, double (&v)[4], bool wide) {
+  if (wide) {
+    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+                 : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
+                 : "l"(p));
+  } else {
+    double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+  }
+}
 
 // Each connection's mass flux a -> b (a < b) per phase, once: upstream
 // mobility (Section 2: Darcy flux with potential Phi = p - rho g z, upstream
@@ -510,7 +555,7 @@ __global__ void __launch_bounds__(kBlock) k_conn_flux(AsmArgs a) {
     double fl = 0.0, pu = up_a ? 0.0 : -0.0, su = up_a ? ms : flip(ms), pd = 0.0;
     double sd = pu;
     // a phase that does not move (residual saturation upstream): all zeros
-    if (capw || ((bits(mob) | bits(mp) | bits(ms)) << 1) != 0) {
+    if (capw || !(is_zero(mob) && is_zero(mp) && is_zero(ms))) {
       const double tm = T * mob;
       fl = tm * dpot;
       if (grav) {
@@ -520,12 +565,12 @@ __global__ void __launch_bounds__(kBlock) k_conn_flux(AsmArgs a) {
         pu = T * ((mp * dpot) + (up_a ? mob : flip(mob)));
         pd = up_a ? flip(tm) : tm;
       }
-      if ((bits(mob) << 1) == 0) pd = 0.0;
+      if (is_zero(mob)) pd = 0.0;
       su = ms * dpot;
       if (capw) {   // - mob p_cow'(a) on a's side, + mob p_cow'(b) on b's
         const double ga = mob * a.pr[9 * n + ia], gb = mob * a.pr[9 * n + ib];
         su = up_a ? su - ga : su + gb;
-        sd = T * (up_a ? ((bits(gb) << 1) == 0 ? 0.0 : gb) : flip(ga));
+        sd = T * (up_a ? (is_zero(gb) ? 0.0 : gb) : flip(ga));
       }
       su = T * su;
     }
@@ -536,12 +581,8 @@ __global__ void __launch_bounds__(kBlock) k_conn_flux(AsmArgs a) {
     fb[2 * al] = up_a ? pd : pu;
     fb[2 * al + 1] = up_a ? sd : su;
   }
-  double2 *oab = reinterpret_cast<double2 *>(a.val + 4 * (size_t)e.x);
-  double2 *oba = reinterpret_cast<double2 *>(a.val + 4 * (size_t)e.y);
-  oab[0] = make_double2(fb[0], fb[1]);
-  oab[1] = make_double2(fb[2], fb[3]);
-  oba[0] = make_double2(fa[0], fa[1]);
-  oba[1] = make_double2(fa[2], fa[3]);
+  store_block(a.val + 4 * (size_t)e.x, fb, a.wide);
+  store_block(a.val + 4 * (size_t)e.y, fa, a.wide);
   a.fconn[c] = make_double2(F[0], F[1]);
 }
 
@@ -639,8 +680,8 @@ __global__ void __launch_bounds__(kBlock) k_assemble(AsmArgs a, int cell_blocks)
   qc.drho[0] = P.drho_o;
   qc.drho[1] = P.drho_w;
   const double phi_ref = mat ? a.phi_m[loc] : a.phi_f[loc];
-  qc.phi = P.c_rock == 0.0 ? phi_ref : phi_ref * (1.0 + P.c_rock * (a.p[r] - P.p_ref_rock));
-  qc.dphi = P.c_rock == 0.0 ? 0.0 : phi_ref * P.c_rock;
+  qc.phi = !P.rock ? phi_ref : phi_ref * (1.0 + P.c_rock * (a.p[r] - P.p_ref_rock));
+  qc.dphi = !P.rock ? 0.0 : phi_ref * P.c_rock;
   double M[2], dM[4];
   accumulation(P, sw, qc, M, dM);
   reinterpret_cast<double2 *>(a.Macc)[r] = make_double2(M[0], M[1]);
@@ -648,36 +689,57 @@ __global__ void __launch_bounds__(kBlock) k_assemble(AsmArgs a, int cell_blocks)
   double r0 = (M[0] - mn.x) * a.inv_dt, r1 = (M[1] - mn.y) * a.inv_dt;
   double d0 = dM[0] * a.inv_dt, d1 = dM[1] * a.inv_dt;
   double d2 = dM[2] * a.inv_dt, d3 = dM[3] * a.inv_dt;
-  // connection c of which this row is cell a (low) or cell b
-  auto conn = [&](size_t c, bool low) {
-    const int2 e = a.cpos[c];
-    const int te = low ? e.y : e.x;
-    if (te < 0) return;
-    const double2 F = a.fconn[c];
-    const double2 *tb = reinterpret_cast<const double2 *>(a.val + 4 * (size_t)te);
-    const double2 t01 = tb[0], t23 = tb[1];
-    r0 = low ? r0 + F.x : r0 - F.x;
-    d0 = d0 - t01.x;
-    if ((bits(t01.y) << 1) != 0) d1 = d1 - t01.y;
-    if (((bits(F.y) | bits(t23.x)) << 1) != 0) {
-      r1 = low ? r1 + F.y : r1 - F.y;
-      d2 = d2 - t23.x;
+  // connection c[q] (none: not there) of which this row is cell a (low) or
+  // cell b: the positions and fluxes of all N first, then their blocks, then
+  // the sums
+  auto conns = [&](auto &c, const auto &there, auto low) {
+    constexpr int N = sizeof(c) / sizeof(c[0]);
+    int te[N];
+    double2 F[N];
+    double tb[N][4];
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      te[q] = -1;
+      if (there[q]) {
+        const int2 e = a.cpos[c[q]];
+        te[q] = low.value ? e.y : e.x;
+        F[q] = a.fconn[c[q]];
+      }
     }
-    if ((bits(t23.y) << 1) != 0) d3 = d3 - t23.y;
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (te[q] >= 0) load_block(a.val + 4 * (size_t)te[q], tb[q], a.wide);
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      if (te[q] < 0) continue;
+      r0 = low.value ? r0 + F[q].x : r0 - F[q].x;
+      d0 = d0 - tb[q][0];
+      if (!is_zero(tb[q][1])) d1 = d1 - tb[q][1];
+      if (!(is_zero(F[q].y) && is_zero(tb[q][2]))) {
+        r1 = low.value ? r1 + F[q].y : r1 - F[q].y;
+        d2 = d2 - tb[q][2];
+      }
+      if (!is_zero(tb[q][3])) d3 = d3 - tb[q][3];
+    }
   };
   const size_t nL = (size_t)P.nL;
   if (mat) {
-    conn(3 * nL + loc, false);
+    const size_t c[1] = {3 * nL + loc};
+    const bool there[1] = {true};
+    conns(c, there, std::false_type{});
   } else {
     int i, j, k;
     loc_ijk(P, loc, i, j, k);
-    if (k > 0) conn(2 * nL + loc - P.nx * P.ny, false);
-    if (j > 0) conn(nL + loc - P.nx, false);
-    if (i > 0) conn((size_t)loc - 1, false);
-    conn(3 * nL + loc, true);
-    if (i < P.nx - 1) conn((size_t)loc, true);
-    if (j < P.ny - 1) conn(nL + loc, true);
-    if (k < P.nz - 1) conn(2 * nL + loc, true);
+    {
+      const size_t c[3] = {2 * nL + loc - (size_t)P.nx * P.ny, nL + loc - P.nx, (size_t)loc - 1};
+      const bool there[3] = {k > 0, j > 0, i > 0};
+      conns(c, there, std::false_type{});
+    }
+    {
+      const size_t c[4] = {3 * nL + loc, (size_t)loc, nL + loc, 2 * nL + loc};
+      const bool there[4] = {true, i < P.nx - 1, j < P.ny - 1, k < P.nz - 1};
+      conns(c, there, std::true_type{});
+    }
     // the perforations come after all cells
     const int cells = 2 + (i > 0) + (j > 0) + (k > 0) + (i < P.nx - 1) + (j < P.ny - 1) +
                       (k < P.nz - 1);
@@ -693,9 +755,8 @@ __global__ void __launch_bounds__(kBlock) k_assemble(AsmArgs a, int cell_blocks)
       off[0] = -dqb[0]; off[1] = 0.0; off[2] = -dqb[1]; off[3] = 0.0;
     }
   }
-  double2 *dg = reinterpret_cast<double2 *>(a.val + 4 * (size_t)a.diag[r]);
-  dg[0] = make_double2(d0, d1);
-  dg[1] = make_double2(d2, d3);
+  const double dg[4] = {d0, d1, d2, d3};
+  store_block(a.val + 4 * (size_t)a.diag[r], dg, a.wide);
   reinterpret_cast<double2 *>(a.R)[r] = make_double2(r0, r1);
 }
 
@@ -805,6 +866,7 @@ int phys_assemble(Sim *s) {
   a.val = s->A.val; a.R = s->R;
   a.fconn = reinterpret_cast<double2 *>(s->fconn);
   a.inv_dt = s->inv_dt;
+  a.wide = ((uintptr_t)s->A.val & 31) == 0;
   void (*k_conn_flux_sel)(AsmArgs) =
       cap ? (grav ? k_conn_flux<true, true> : k_conn_flux<false, true>)
           : (grav ? k_conn_flux<true, false> : k_conn_flux<false, false>);
@@ -828,7 +890,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 
 // max of non-negative doubles as integers (a NaN counts as 0, as fmax drops it)
 __device__ __forceinline__ long long max_bits(double v) {
-  long long b = bits(v) & 0x7fffffffffffffffll;
+  long long b = __double_as_longlong(v) & 0x7fffffffffffffffll;
   return b > 0x7ff0000000000000ll ? 0 : b;
 }
 __device__ __forceinline__ double warp_max_bits(long long b) {

@@ -236,6 +236,7 @@ extern "C" int sim_create(const dp_grid *grid, const dp_rock *rock, const dp_flu
   P.sigma = rock->sigma; P.c_rock = rock->c_rock; P.p_ref_rock = rock->p_ref;
   P.drho_o = fluid->rho_o_ref * fluid->c_o;   // the products props() forms, once
   P.drho_w = fluid->rho_w_ref * fluid->c_w;
+  P.rock = rock->c_rock != 0.0;
   auto fail = [&](int rc) { sim_destroy(s); return rc; };
   for (int k = 0; k < 2; ++k) {
     P.pc_n[k] = fluid->pc_n[k];
