@@ -752,7 +752,6 @@ int level_dinv(Sim *s, Level &L) {
 
 static int level_prepare(Sim *s, Level &L) {
   int n = L.n;
-  L.G = lanes_for(n > 0 ? (double)L.nnz / n : 0.0);
   L.dpos = (int *)dalloc(s, (size_t)n * 4);
   L.tpos = (int *)dalloc(s, (size_t)std::max(L.nnz, 1) * 4);
   L.colour = (int *)dalloc(s, (size_t)n * 4);
@@ -786,6 +785,9 @@ static int level_prepare(Sim *s, Level &L) {
     DP_TRY(greedy_colour(s, n, L.rowptr, L.col, L.colour, &L.ncolour));
     DP_TRY(colour_lists(s, n, L.colour, L.ncolour, L.clist, L.cstart, nullptr));
   }
+  // rows of a launch: the level's, or with Gauss-Seidel a colour's
+  L.G = cycle_lanes(0, s->opt.precision == 0, L.l1 ? n : (double)n / std::max(L.ncolour, 1),
+                    n > 0 ? (double)L.nnz / n : 0.0);
   return DP_OK;
 }
 
@@ -947,8 +949,8 @@ int amg_setup(Sim *s) {
     N.dinv = (double *)dalloc(s, (size_t)std::max(na, 1) * 8);
     N.dinvf = (float *)dalloc(s, (size_t)std::max(na, 1) * 4);
     if (!N.dinv || !N.dinvf) { s->fail(DP_ENOMEM, "allocation failed"); return DP_ENOMEM; }
-    L.p_G = lanes_for((double)L.p_nnz / n);
-    L.r_G = lanes_for((double)L.p_nnz / na);
+    L.p_G = cycle_lanes(2, o.precision == 0, n, (double)L.p_nnz / n);
+    L.r_G = cycle_lanes(1, o.precision == 0, na, (double)L.p_nnz / na);
     N.val = (double *)dalloc(s, (size_t)std::max(N.nnz, 1) * 8);
     N.valf = (float *)dalloc(s, (size_t)std::max(N.nnz, 1) * 4);
     if (!L.ap_val || !N.val || !N.valf) { s->fail(DP_ENOMEM, "allocation failed"); return DP_ENOMEM; }

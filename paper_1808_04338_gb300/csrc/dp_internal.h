@@ -261,6 +261,7 @@ int la_alloc(Sim *s);
 int mixed_refresh(Sim *s, bool coarse);
 int l0_refresh(Sim *s, bool coarse);
 int lanes_for(double mean_len);
+int cycle_lanes(int op, bool f64, double rows, double len);
 void graphs_free(Sim *s);
 int autotune(Sim *s, int reps, std::string &report);
 
@@ -390,7 +391,11 @@ struct Sim {
   double *p0c_val = nullptr, *dinv_c = nullptr;
   float *p0c_valf = nullptr, *dinv_cf = nullptr;
   bool l0_lu = false;
-  int l0_G = 1;       // lanes per row of the level-0 colour-order sweeps (autotuned; 1: a thread)
+  // the kernel of the level-0 colour-order sweeps and residual
+  // (sim_set_l0_kernel): the pipelined one was the fastest or within 2% of it
+  // from 5765 rows (two sweeps and a residual 12.5 us, a thread per row 15.5)
+  // to 4M (128 and 155), in FP64 too (200005 rows: 32.7 and 45.2)
+  int l0_G = -1;
   int shapes = 0;     // bumped whenever launch shapes change (autotune, AMG set-up)
   double *l0_pv = nullptr;
   float *l0_pvf = nullptr;   // inverse from the LU factors (n <= kInverseMax), row-major

@@ -1021,13 +1021,33 @@ __global__ void __launch_bounds__(kBlock) k_csr_resid(int n, const int *__restri
 }
 
 
-// Lanes per row for a mean row length: enough lanes that each walks about
-// eight entries (two rounds of four loads in flight), no more, because on
-// GB300 FP64 issue is scarce (1.2 TFLOP/s for the whole GPU) and every lane
-// of a group takes part in the log2(G) shuffle additions.
+// Lanes per row of the set-up's products for a mean row length: enough lanes
+// that each walks about eight entries.
 int lanes_for(double mean_len) {
   int g = 1;
   while (g < 32 && 8.0 * g < mean_len) g *= 2;
+  return g;
+}
+
+// Lanes per row of a level's V-cycle kernels (op 0 the operator, 1 the
+// restriction, 2 the prolongation) for `rows` rows a launch of mean length
+// `len`.  A coarse level's launch is a chain of dependent loads, so a lane
+// takes one or two entries; that many lanes fill the GPU and then cost, in
+// FP64 sooner (the lanes' reduction adds take the SM's two FP64 lanes a
+// cycle), so the threads of a launch are capped.  The caps lie where the
+// autotuner's timings turn, FP32 on levels of 568928, 87367, 13601, 2012 rows:
+// operator 4, 16, 32, 32 lanes (10.1 us on the second instead of 12.4 at 8,
+// 2.4 on the last instead of 3.6 at 16), restriction 2, 8, 16, 16 (2.4 us into
+// the third instead of 3.9 at 4); FP64 on 144677, 22225, 3411 rows: operator
+// 2, 4, 16 (17.4, 9.0 and 4.5 us; with 4, 8 and 16 21.7, 10.9 and 4.5).
+int cycle_lanes(int op, bool f64, double rows, double len) {
+  double per = f64 ? (op == 0 || op == 2 ? 2.0 : 1.0) : (op == 0 ? 1.6 : 1.0);
+  double cap = f64 ? (op == 2 ? 6.0e4 : 9.0e4) : (op == 0 ? 2.5e6 : op == 1 ? 1.2e6 : 2.0e5);
+  int lo = f64 && op == 0 && len > 8.0 ? 2 : 1, g = 1;
+  while (g < 32 && per * g < len) g *= 2;
+  if (!f64 && op == 0 && g > 1 && 2.5 * g > 2.0 * len) g /= 2;
+  while (g > lo && rows * g > cap) g /= 2;
+  while (!f64 && op == 0 && g < 32 && g < len && rows * g <= 8192.0) g *= 2;
   return g;
 }
 
