@@ -27,6 +27,7 @@ UNITS = {
     "dp_sim.cu": [],
     "dp_noalloc.cu": [],
     "dp_cycle.cu": [],
+    "dp_small.cu": [],
     "dp_serve.cu": [],
     "dp_batch.cu": [],
 }
@@ -50,7 +51,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
     nvcc = _nvcc()
     headers = [os.path.join(CSRC, "dp_internal.h"), os.path.join(CSRC, "dp_kernels.cuh"),
-               os.path.join(ROOT, "include", "dpsim.h")]
+               os.path.join(CSRC, "dp_tma.cuh"), os.path.join(ROOT, "include", "dpsim.h")]
     jobs = []
     objs = []
     for src, extra in UNITS.items():

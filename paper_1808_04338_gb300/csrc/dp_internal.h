@@ -265,6 +265,17 @@ int cycle_lanes(int op, bool f64, double rows, double len);
 void graphs_free(Sim *s);
 int autotune(Sim *s, int reps, std::string &report);
 
+// dp_small.cu (the CPR-FPF phases around the V-cycle in one cluster launch
+// each, small realisations): part 0 before it, part 1 after it
+struct X0Init;
+bool cpr_small(const Sim *s);
+template <typename T>
+int cpr_small_part(Sim *s, int part, const double *r, double *z, const int *omap,
+                   const X0Init &xi, bool colour_z);
+// and the product, Gram-Schmidt and Givens rotations of an Arnoldi step
+bool orth_small(const Sim *s);
+int orth_small_step(Sim *s, int j, const double *z, double *vnext);
+
 // dp_cycle.cu (the coarse levels of the V-cycle in one cluster launch)
 constexpr int kClusterMaxRows = 20000;   // default of dp_options.cluster_rows
 int cluster_setup(Sim *s);

@@ -2709,6 +2709,12 @@ int cpr_apply(Sim *s, const double *r, double *z) {
   }
   if (!f32) {
     if (s->opt.precond == 1) return ilu_apply(s, r, z);
+    if (cpr_small(s)) {   // the phases around the V-cycle in a cluster launch each
+      const int *m = l0c_on(s) ? s->iperm : nullptr;
+      DP_TRY(cpr_small_part<double>(s, 0, r, z, m, X0Init(), false));
+      DP_TRY(vcycle(s, 0, s->rp, s->xp));
+      return cpr_small_part<double>(s, 1, r, z, m, X0Init(), false);
+    }
     DP_TRY(ilu_apply(s, r, s->z1));
     const int *m = l0c_on(s) ? s->iperm : nullptr;   // level-0 vectors in colour order
     DP_LAUNCH_PDL(s, kPdlSmall, k_bsr_presid, 1 + nblk(s->sv_long0), kBlock, 0, nb, s->sv_sL, s->sv_sc,
@@ -2730,7 +2736,8 @@ int cpr_apply(Sim *s, const double *r, double *z) {
   // the final sum; the second application writes s->ilu_zp2), or, when level
   // 0 is not in colour order, gathered into natural order (z1f)
   Level &L0 = s->lev[0];
-  DP_TRY((ilu_apply_t<float, double>(s, s->lu_valf, r)));
+  const bool small = cpr_small(s);
+  if (!small) DP_TRY((ilu_apply_t<float, double>(s, s->lu_valf, r)));
   const int *m = l0c_on(s) ? s->iperm : nullptr;     // level-0 vectors in colour order
   // with level 0 in colour order, z1 stays in the ILU(0) colour order: the
   // stage residuals gather it, and z2, there through the colour positions
@@ -2739,7 +2746,7 @@ int cpr_apply(Sim *s, const double *r, double *z) {
   bool cz = m && s->scolc && s->z2c;
   const float *z1s = cz ? reinterpret_cast<const float *>(s->ilu_zp) : s->z1f;
   const int *scs = cz ? s->scolc : s->scol;
-  if (!cz) DP_TRY(ilu_result<float>(s, nullptr, nullptr, s->z1f));
+  if (!cz && !small) DP_TRY(ilu_result<float>(s, nullptr, nullptr, s->z1f));
   X0Init xi;   // in colour order, the pre-smoothing's start written with b
   if (m) {
     int f = 0;
@@ -2750,6 +2757,11 @@ int cpr_apply(Sim *s, const double *r, double *z) {
       xi.f0 = s->lu_cstart[f];
       xi.f1 = s->lu_cstart[f + 1];
     }
+  }
+  if (small) {   // the phases around the V-cycle in a cluster launch each
+    DP_TRY(cpr_small_part<float>(s, 0, r, z, m, xi, cz));
+    DP_TRY(vcycle_t<float>(s, 0, L0.bf, L0.xf, xi.x != nullptr));
+    return cpr_small_part<float>(s, 1, r, z, m, xi, cz);
   }
   DP_LAUNCH_PDL(s, kPdlSmall, k_bsr_presid_f32, 1 + nblk(s->sv_long0), kBlock, 0, nb, s->sv_sL, s->sv_sc,
             s->sv_long0, s->srowptr, scs, reinterpret_cast<const float2 *>(s->spf), z1s, r, L0.bf,
@@ -2912,6 +2924,7 @@ static int arnoldi_step(Sim *s, int j) {
   double *vj = s->V + (long long)j * N, *zj = s->Z + (long long)j * N;
   double *vnext = s->V + (long long)(j + 1) * N;
   DP_TRY(cpr_apply(s, vj, zj));
+  if (orth_small(s)) return orth_small_step(s, j, zj, vnext);
   DP_TRY(bsr_spmv(s, zj, s->w));
   DP_TRY(dots(s, s->V, N, j + 1, s->w, 3, j));
   DP_LAUNCH_PDL(s, kPdlSmall, k_project, gridN, kBlock, 0, N, s->V, N, j + 1, s->dots, s->w, vnext, s->scal, 0, small_trig(s));

@@ -118,3 +118,35 @@ def test_assembly_with_resting_phases_bit_exact(gravity, capillary, swc_fraction
         out.append(s.jacobian())
     for g, o in zip(out[0][2:], out[1][2:]):
         assert np.array_equal(g.view(np.uint64), o.view(np.uint64))
+
+
+def few(prob, its, kw, state):
+    """(iterations, relative residual, update) of one solve of at most `its` iterations."""
+    s = gpu().Sim(prob, gpu().options("parity", eta_fixed=1e-13, gmres_maxit=its, **kw))
+    s.set_iterate(*state)
+    s.assemble(prob.dt)
+    _, st = s.solve_step()
+    return st.linear_iters, st.lin_relres
+
+
+# the cluster launches of a small realisation against one launch a phase
+# (cluster_rows < 0): a location, no wells, a well of short rows and of long
+# rows (more than 24 blocks), the last size that takes them (8192 rows) and
+# the next, restarts, one and two Gram-Schmidt passes, precisions, the
+# eliminated system
+@pytest.mark.parametrize("grid,wells", [((1, 1, 1), "bhp"), ((9, 1, 1), "none"), ((7, 5, 3), "two"),
+                                        ((6, 5, 40), "two"), ((64, 64, 1), "none"),
+                                        ((64, 64, 1), "bhp"), ((17, 16, 15), "two")])
+@pytest.mark.parametrize("kw", [{}, dict(gmres_restart=3, reorth=1e-10), dict(schur=1),
+                                dict(precision=1, amg_gs_levels=1), dict(precision=1, schur=1),
+                                dict(precision=1, reorth=2.0, amg_coarse_max=16)])
+def test_small_preconditioner_and_arnoldi_step(grid, wells, kw):
+    prob = small(*grid, wells=wells)
+    state = interior(prob, 3)
+    its, r = few(prob, 5, kw, state)
+    its0, r0 = few(prob, 5, dict(kw, cluster_rows=-1), state)
+    assert its == its0
+    # FP64: rounding; FP32 preconditioner: its 24 bits, through five iterations
+    # (a residual at the floor of the system's conditioning agrees in size only)
+    tol = 1e-6 if not kw.get("precision") else 1e-2
+    assert abs(r - r0) <= tol * r0 + 1e-11
