@@ -720,7 +720,7 @@ static int build_plan(dp_batch *b) {
     Sim *s = b->m[k];
     long long N = 2LL * s->K.n;
     Ns[k] = N;
-    gridN[k] = (int)std::min<long long>(nblk(N), kDotBlocks * 4);
+    gridN[k] = (int)std::min<long long>(nblk(N / 2), kDotBlocks * 4);   // pairs
     gridNb[k] = nblk(N);
     dotg[k] = dot_blocks(N);
   }

@@ -12,6 +12,26 @@
 
 namespace dp {
 
+// FP64 to FP32 (to nearest even) on the integer pipe: GB300 converts on the
+// FP64 pipe, where an instruction holds a quarter of the SM for 64 cycles.
+// The conversion instruction's value, bit for bit; numbers outside FP32's
+// normal range take the instruction.  Only where conversions are what bounds
+// a kernel (k_decouple, 200 x 200 x 50 cells: 457 -> 424 us); the gather-bound ones gained nothing.
+__device__ __forceinline__ float narrow(double v) {
+  const unsigned h = (unsigned)__double2hiint(v), l = (unsigned)__double2loint(v);
+  const unsigned m = h & 0x7fffffffu;
+  if ((m | l) == 0u) return __uint_as_float(h);
+  if (m < 0x38100000u || m >= 0x47e00000u) return float(v);   // below 2^-126 or from 2^127 on
+  unsigned r = ((m - 0x38000000u) << 3) | (l >> 29);
+  const unsigned rem = l & 0x1fffffffu;
+  r += rem > 0x10000000u || (rem == 0x10000000u && (r & 1u)) ? 1u : 0u;
+  return __uint_as_float((h & 0x80000000u) | r);
+}
+template <typename T, typename TR> __device__ __forceinline__ T narrow_to(TR v) {
+  if constexpr (sizeof(T) < sizeof(TR)) return narrow(v);
+  else return T(v);
+}
+
 constexpr int kLongRow = 24;   // colours with a row longer than this use a warp per row
 
 // The well rows (storage rows nlong..n-1, one block per perforation, tens of
@@ -1097,12 +1117,35 @@ __device__ __forceinline__ void k_project_b(int bx, int gx, long long N, const d
   if (threadIdx.x < nv) cs[threadIdx.x] = -c[threadIdx.x];
   __syncthreads();
   if (fin < 0) return;
-  for (long long i = (long long)bx * blockDim.x + threadIdx.x; i < N;
+  // Pairs of elements (N is even), four basis vectors' loads in flight: bound
+  // by the basis read once.  200 x 200 x 50 cells, mean of a step's launches:
+  // 67.0 -> 64.3 us.  The grid counts pairs: with idle CTAs left in it sixteen
+  // small models in lockstep took 51.85 ms a step, 50.82 without.
+  const long long N2 = N >> 1, ld2 = ldv >> 1;
+  const double2 *V2 = reinterpret_cast<const double2 *>(V);
+  double2 *w2 = reinterpret_cast<double2 *>(w);
+  double2 *o2 = reinterpret_cast<double2 *>(out);
+  for (long long i = (long long)bx * blockDim.x + threadIdx.x; i < N2;
        i += (long long)gx * blockDim.x) {
-    double acc = w[i];
-    for (int k = 0; k < nv; ++k) acc = fma(cs[k], V[k * ldv + i], acc);
-    if (fin) out[i] = acc * rb;
-    else w[i] = acc;
+    double2 acc = w2[i];
+    int k = 0;
+    for (; k + 4 <= nv; k += 4) {
+      double2 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = __ldg(V2 + (k + u) * ld2 + i);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        acc.x = fma(cs[k + u], v[u].x, acc.x);
+        acc.y = fma(cs[k + u], v[u].y, acc.y);
+      }
+    }
+    for (; k < nv; ++k) {
+      double2 v = __ldg(V2 + k * ld2 + i);
+      acc.x = fma(cs[k], v.x, acc.x);
+      acc.y = fma(cs[k], v.y, acc.y);
+    }
+    if (fin) o2[i] = make_double2(acc.x * rb, acc.y * rb);
+    else w2[i] = acc;
   }
 }
 
@@ -1113,11 +1156,19 @@ __device__ __forceinline__ void k_multi_axpy_b(int bx, int gx, long long N, cons
   __shared__ double cs[32];
   if (threadIdx.x < nv) cs[threadIdx.x] = sign * c[threadIdx.x];
   __syncthreads();
-  for (long long i = (long long)bx * blockDim.x + threadIdx.x; i < N;
+  const long long N2 = N >> 1, ld2 = ldv >> 1;
+  const double2 *V2 = reinterpret_cast<const double2 *>(V);
+  double2 *w2 = reinterpret_cast<double2 *>(w);
+  for (long long i = (long long)bx * blockDim.x + threadIdx.x; i < N2;
        i += (long long)gx * blockDim.x) {
-    double acc = w[i];
-    for (int k = 0; k < nv; ++k) acc += cs[k] * V[k * ldv + i];
-    w[i] = acc;
+    double2 acc = w2[i];
+#pragma unroll 4
+    for (int k = 0; k < nv; ++k) {
+      double2 v = __ldg(V2 + k * ld2 + i);
+      acc.x = fma(cs[k], v.x, acc.x);
+      acc.y = fma(cs[k], v.y, acc.y);
+    }
+    w2[i] = acc;
   }
 }
 

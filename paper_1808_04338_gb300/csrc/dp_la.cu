@@ -2920,7 +2920,7 @@ __global__ void k_sqrt_inplace(double *v) {
 static int arnoldi_step(Sim *s, int j) {
   int m = s->m;
   long long N = 2LL * s->K.n;
-  int gridN = (int)std::min<long long>(nblk(N), kDotBlocks * 4);
+  int gridN = (int)std::min<long long>(nblk(N / 2), kDotBlocks * 4);   // pairs
   double *vj = s->V + (long long)j * N, *zj = s->Z + (long long)j * N;
   double *vnext = s->V + (long long)(j + 1) * N;
   DP_TRY(cpr_apply(s, vj, zj));
@@ -2992,7 +2992,7 @@ int fgmres(Sim *s, double tol, int *iters, double *relres) {
   bool conv = false;
   double res = bnorm;
   if (bnorm == 0.0) { conv = true; res = 0.0; }
-  int gridN = (int)std::min<long long>(nblk(N), kDotBlocks * 4);
+  int gridN = (int)std::min<long long>(nblk(N / 2), kDotBlocks * 4);   // pairs
   while (!conv && total < maxit) {
     // v_0 = r / ||r||.  The first cycle starts from x = 0, where r = b - A 0
     // = b exactly and ||r|| = ||b|| is already in scal[0]: no product.
