@@ -609,7 +609,7 @@ static void ilu_sweeps(const Sim *s, std::vector<Sweep> &fwd, std::vector<Sweep>
     bool lng = s->lu_cmaxlen[c] > kLongRow;
     if (c == last && lng) continue;
     if (lng) bwd.push_back({1, r0, r1, nblk(32LL * (r1 - r0))});
-    else bwd.push_back({0, r0, r1, nblk((r1 - r0 + kRes - 1) / kRes)});
+    else bwd.push_back({0, r0, r1, nblk((r1 - r0 + kBwdRes<float> - 1) / kBwdRes<float>)});
   }
 }
 

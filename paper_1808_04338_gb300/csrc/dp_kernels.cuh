@@ -98,6 +98,16 @@ template <> struct Blk<double> {
 };
 
 constexpr int kRes = 4;   // rows per thread of the gather-style kernels
+// CTAs of their launch: kRes rows a thread, but as many CTAs as rows allow
+// until eight an SM (kBlock threads each) are resident; a thread steps over
+// rows by the grid, so any grid from rows / kRes up serves.  At four rows a
+// thread a colour of 112k rows is 110 CTAs for 152 SMs.
+// 93 x 71 x 17 cells in BF16: a step 15.63 -> 15.24 ms; 100 x 100 x 10 cells in
+// FP64 84.5 -> 83.3 ms; from 1.25M rows on the grid is the one of four.
+inline int res_blocks(long long rows) {
+  const int few = nblk((rows + kRes - 1) / kRes), fill = 8 * 152;
+  return few >= fill ? few : (int)(nblk(rows) < fill ? nblk(rows) : fill);
+}
 
 // Warp-per-row variants of the sweeps for colours with long rows (the well
 // rows, one entry per perforation): the lanes split the row's blocks and
@@ -467,6 +477,11 @@ __device__ __forceinline__ void k_ilu_fwd_copy_b(int bx, int gx, int r0, int r1,
   }
 }
 
+// Rows per thread of the backward sweep: with FP64 blocks four rows' pivots
+// and sums leave too few warps in flight for the gathers.  One row a thread:
+// 121 x 113 x 37 cells, a solve 23.61 -> 23.23 ms; 100 x 100 x 10 cells, a step
+// 83.3 -> 82.5 ms.  FP32 takes res_blocks.
+template <typename T> constexpr int kBwdRes = sizeof(T) == 8 ? 1 : kRes;
 template <typename T>
 __device__ __forceinline__ void k_ilu_bwd_r_b(int bx, int gx, int r0, int r1, int nL, int n,
                                                       const int *__restrict__ Uptr,
@@ -477,11 +492,11 @@ __device__ __forceinline__ void k_ilu_bwd_r_b(int bx, int gx, int r0, int r1, in
   size_t ub = (size_t)nL + n;
   int S = gx * blockDim.x;
   int q0 = r0 + bx * blockDim.x + threadIdx.x;
-  int ea[kRes], eb[kRes];
-  T d[kRes][4];
-  T2 y[kRes];
+  int ea[kBwdRes<T>], eb[kBwdRes<T>];
+  T d[kBwdRes<T>][4];
+  T2 y[kBwdRes<T>];
 #pragma unroll
-  for (int k = 0; k < kRes; ++k) {
+  for (int k = 0; k < kBwdRes<T>; ++k) {
     int q = q0 + k * S;
     bool ok = q < r1;
     ea[k] = ok ? __ldcs(Uptr + q) : 0;
@@ -492,7 +507,7 @@ __device__ __forceinline__ void k_ilu_bwd_r_b(int bx, int gx, int r0, int r1, in
     }
   }
 #pragma unroll
-  for (int k = 0; k < kRes; ++k) {
+  for (int k = 0; k < kBwdRes<T>; ++k) {
     int q = q0 + k * S;
     if (q >= r1) continue;
     T s0 = T(0), s1 = T(0);

@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(kBlock) k_ilu_fwd_copy(int r0, int r1, const i
 }
 
 // Backward sweep of one colour (short rows): zp_r = D_r (zp_r - sum_{U}
-// U_rj zp_j) with D_r the inverted pivot; a thread per row, kRes rows per
+// U_rj zp_j) with D_r the inverted pivot; a thread per row, kBwdRes rows per
 // thread, each row's pivot block and y loaded with its U pointers before the
 // U gathers (a two-lanes-per-row version, one output component a lane, was
 // 2% slower on the cell colours and 2.3 times slower on the colour before
@@ -752,7 +752,7 @@ static int ilu_apply_t(Sim *s, const T *lu, const TR *r, T *zpo = nullptr) {
       DP_LAUNCH_PDL(s, kPdlSmall, (k_ilu_fwd_w<T, TR, false>), nblk(32LL * (r1 - r0)), kBlock, 0, r0, r1, nL,
                 s->perm, s->lu_Lptr, s->lu_colp, lu, r, zp, small_trig(s));
     else if (c == first)   // no L blocks
-      DP_LAUNCH_PDL(s, kPdlSmall, (k_ilu_fwd_copy<T, TR>), nblk((r1 - r0 + kRes - 1) / kRes), kBlock, 0, r0, r1,
+      DP_LAUNCH_PDL(s, kPdlSmall, (k_ilu_fwd_copy<T, TR>), res_blocks(r1 - r0), kBlock, 0, r0, r1,
                 s->perm, r, zp, small_trig(s));
     else
       DP_LAUNCH_PDL(s, kPdlSmall, (k_ilu_fwd<T, TR>), nblk(2LL * (r1 - r0)), kBlock, 0, r0, r1, s->perm,
@@ -768,7 +768,8 @@ static int ilu_apply_t(Sim *s, const T *lu, const TR *r, T *zpo = nullptr) {
       DP_LAUNCH_PDL(s, kPdlSmall, k_ilu_bwd_w<T>, nblk(32LL * (r1 - r0)), kBlock, 0, r0, r1, nL, n,
                 s->lu_Uptr, s->lu_colp, lu, zp, small_trig(s));
     else
-      DP_LAUNCH_PDL(s, kPdlSmall, k_ilu_bwd_r<T>, nblk((r1 - r0 + kRes - 1) / kRes), kBlock, 0, r0, r1, nL, n,
+      DP_LAUNCH_PDL(s, kPdlSmall, k_ilu_bwd_r<T>,
+                    kBwdRes<T> == kRes ? res_blocks(r1 - r0) : nblk(r1 - r0), kBlock, 0, r0, r1, nL, n,
                 s->lu_Uptr, s->lu_colp, lu, zp, small_trig(s));
   }
   return DP_OK;
@@ -804,7 +805,7 @@ static int ilu_result(Sim *s, const double *base, double *out, T *outT = nullptr
                       const float *inj = nullptr, int inj_perm = 0, const T *zb = nullptr,
                       const T *zp = nullptr) {
   int n = s->K.n;
-  DP_LAUNCH_PDL(s, kPdlSmall, k_ilu_result<T>, nblk((n + kRes - 1) / kRes), kBlock, 0, n, s->iperm,
+  DP_LAUNCH_PDL(s, kPdlSmall, k_ilu_result<T>, res_blocks(n), kBlock, 0, n, s->iperm,
             zp ? zp : reinterpret_cast<const T *>(s->ilu_zp), base, out, outT, inj, inj_perm, zb, small_trig(s));
   return DP_OK;
 }

@@ -178,3 +178,18 @@ def test_batch_rejects_unsupported_members():
         h = C.c_void_p()
         assert L.batch_create(C.cast(H, C.c_void_p), 1, None, C.byref(h)) == gpu().DP_EINVAL, kw
         s.close()
+
+
+# rows of a colour: one below, at and above eight CTAs an SM (1216 x 256), and
+# a remainder on either side
+@pytest.mark.parametrize("nx,ny,nz", [(131, 113, 21), (128, 128, 19), (129, 97, 25)])
+def test_sweep_grids_equal_bit_for_bit(nx, ny, nz):
+    """The ILU sweeps of a sim alone spread their rows over as many CTAs as
+    are resident, a batch's take four rows a thread: the same values."""
+    members = [di.layered(nx=nx, ny=ny, nz=nz)]
+    opts = gpu().options("report", precision=1, cluster_rows=-1)
+    a = _alone_run(members, opts, 1)[0][0]
+    m = _batch_run(members, opts, 1)[0][0][0]
+    assert a[:3] == m[:3]
+    for x, y in zip(a[3], m[3]):
+        np.testing.assert_array_equal(x, y)
