@@ -407,6 +407,7 @@ struct Sim {
   // from 5765 rows (two sweeps and a residual 12.5 us, a thread per row 15.5)
   // to 4M (128 and 155), in FP64 too (200005 rows: 32.7 and 45.2)
   int l0_G = -1;
+  bool l0_chosen = false;   // by sim_set_l0_kernel or sim_autotune: see l0_share
   int shapes = 0;     // bumped whenever launch shapes change (autotune, AMG set-up)
   double *l0_pv = nullptr;
   float *l0_pvf = nullptr;   // inverse from the LU factors (n <= kInverseMax), row-major

@@ -55,6 +55,7 @@ struct dp_server {
   std::unordered_map<int64_t, dp_srv_result> done;
   std::vector<std::thread> workers;
   bool stop = false;
+  bool several = false;   // more than one worker
   dp_options opts{};
   int device = 0;
   uint64_t budget = 0, resident_bytes = 0, peak_resident = 0;
@@ -177,6 +178,8 @@ void dp_server::worker() {
         r.rock.phi_f = r.phi_f.data(); r.rock.phi_m = r.phi_m.data();
         rc = sim_create(&r.grid, &r.rock, &r.fluid, r.wells.data(), (int32_t)r.wells.size(),
                         &opts, nullptr, (void *)r.stream, &r.sim);
+        // the level-0 kernel for a GPU that several streams share
+        if (rc == DP_OK && several) rc = sim_set_l0_kernel(r.sim, 1);
         if (rc == DP_OK) rc = sim_set_state(r.sim, r.p.data(), r.sw.data(), r.bhp.data());
       }
     }
@@ -235,6 +238,7 @@ extern "C" int srv_create(int32_t workers, uint64_t hbm_budget, const dp_options
   }
   s->opts = *opts;
   s->budget = hbm_budget;
+  s->several = workers > 1;
   try {
     for (int w = 0; w < workers; ++w) s->workers.emplace_back([s] { s->worker(); });
   } catch (...) {
