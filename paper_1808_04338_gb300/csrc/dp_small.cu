@@ -495,6 +495,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_orth_small(const OrthArgs 
   const long long N = 2LL * A.n;
   const int chunk = (int)((N + 2 * C - 1) / (2 * C)) * 2;
   const int lo = min(rank * chunk, (int)N), len = min(chunk, (int)N - lo), nv = A.j + 1;
+  small_arrive();   // waited for before the first store to another CTA's shared memory
   griddep_wait();
   if (trig) griddep_launch_dependents();
   {   // w = A z over the slice's rows, as k_bsr_spmv_b<0>
@@ -531,6 +532,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_orth_small(const OrthArgs 
     }
   }
   __syncthreads();
+  small_wait();   // every CTA of the cluster has started: its shared memory may be written
   for (int pass = 0; pass < 2; ++pass) {
     for (int k = warp; k <= nv; k += nw) {   // a warp per vector (nv: w itself)
       const double *v = A.V + (k < nv ? k : 0) * N + lo;
