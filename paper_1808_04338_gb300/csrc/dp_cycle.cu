@@ -185,19 +185,23 @@ struct CsrHead {
 };
 
 // One phase over the rows of a CSR operator: s_i = sum_j a_ij X(j), then
-// done(i, s_i, lane of the group) on every lane of the row's group.
-template <typename T, typename F, typename D>
+// done(i, s_i, o_i, lane of the group) on every lane of the row's group.
+// o_i = own(i) is what the row reads of its own entry: every lane has read it
+// before any lane stores, as a put writes this CTA's copy too.
+template <typename T, typename F, typename O, typename D>
 __device__ __forceinline__ void csr_phase(int count, int G, int rank, int C,
                                           const int *__restrict__ rowptr,
                                           const int *__restrict__ col, const T *__restrict__ val,
-                                          F X, D done) {
+                                          F X, O own, D done) {
   RowMap m(G, count, rank, C);
   CsrHead<T> h;
   if (m.any) h.load(m.q < count, m.q, m.gl, G, rowptr, col, val);
   cl_wait();
   while (m.any) {
+    const T o = m.q < count ? own(m.q) : T(0);
     T s = group_reduce<T>(h.dot(G, col, val, X), G);
-    if (m.q < count) done(m.q, s, m.gl);
+    __syncwarp();
+    if (m.q < count) done(m.q, s, o, m.gl);
     if (m.next(count)) h.load(m.q < count, m.q, m.gl, G, rowptr, col, val);
   }
   cl_arrive();
@@ -281,6 +285,7 @@ __device__ void gs_sweep_cl(const LevelDev<T> &Ld, const VB b, const Rep<T> x, b
         s = fma(ve.y, x.get(ce.y), s);
       }
       s = group_reduce<T>(s, G);
+      __syncwarp();   // xi is read on every lane before a put writes this CTA's copy
       if (m.q < ncr && !is_zero(di)) x.put(i, fma(-s, di, xi), m.gl, G, C);
       if (m.next(ncr)) load();
     }
@@ -370,9 +375,8 @@ __device__ void jacobi_post_cl(const LevelDev<T> &L, const VB b, const Rep<T> x,
   const T *__restrict__ d = L.dinv;
   csr_phase<T>(
       L.n, G, rank, C, L.rowptr, L.col, L.val, [&](int c) { return x.get(c); },
-      [&](int i, T s, int gl) {
-        t.put(i, fma(b.get(i) - s, __ldg(d + i), x.get(i)), gl, G, C);
-      });
+      [&](int i) { return x.get(i); },
+      [&](int i, T s, T o, int gl) { t.put(i, fma(b.get(i) - s, __ldg(d + i), o), gl, G, C); });
 }
 
 // x = inv b for the coarsest level from its explicit FP64 inverse: one phase
@@ -455,12 +459,13 @@ __global__ void __launch_bounds__(kClusterThreads, 1)
       const int G = L.lanes;
       csr_phase<T>(
           L.n, G, rank, C, L.rowptr, L.col, L.val, [&](int c) { return x.get(c); },
-          [&](int i, T s, int gl) { r.put(i, b.get(i) - s, gl, G, C); });
+          [&](int i) { return b.get(i); },
+          [&](int i, T s, T o, int gl) { r.put(i, o - s, gl, G, C); });
     }
     const int rG = L.r_lanes;
     csr_phase<T>(
         L.nn, rG, rank, C, L.r_rowptr, L.r_col, L.r_val, [&](int c) { return r.get(c); },
-        [&](int I, T s, int gl) { nb.put(I, s, gl, rG, C); });
+        [](int) { return T(0); }, [&](int I, T s, T, int gl) { nb.put(I, s, gl, rG, C); });
   }
   // coarsest level; in_r: a level's result is in its r (after an l1-Jacobi
   // post-smoothing), else in its x
@@ -492,13 +497,16 @@ __global__ void __launch_bounds__(kClusterThreads, 1)
     const Rep<T> x = xv(l), nx = xv(l + 1);
     const VB b = bv(l), r = rv(l), nr = rv(l + 1);
     const int pG = L.p_lanes;
-    auto add = [&](int i, T s, int gl) { x.put(i, x.get(i) + s, gl, pG, C); };
+    auto own = [&](int i) { return x.get(i); };
+    auto add = [&](int i, T s, T o, int gl) { x.put(i, o + s, gl, pG, C); };
     if (in_r)
       csr_phase<T>(
-          L.n, pG, rank, C, L.p_rowptr, L.p_col, L.p_val, [&](int c) { return nr.get(c); }, add);
+          L.n, pG, rank, C, L.p_rowptr, L.p_col, L.p_val, [&](int c) { return nr.get(c); },
+          own, add);
     else
       csr_phase<T>(
-          L.n, pG, rank, C, L.p_rowptr, L.p_col, L.p_val, [&](int c) { return nx.get(c); }, add);
+          L.n, pG, rank, C, L.p_rowptr, L.p_col, L.p_val, [&](int c) { return nx.get(c); },
+          own, add);
     in_r = L.l1;
     if (L.l1) jacobi_post_cl<T>(L, b, x, r, rank, C);
     else gs_sweep_cl<T>(L, b, x, false, rank, C);

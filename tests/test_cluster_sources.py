@@ -54,3 +54,22 @@ __global__ void k_fine(float *x) {
 }
 """
     assert unsynchronised(src) == ["k_early"]
+
+
+def own_entry_stores(text):
+    """Stores to a replicated vector whose value reads that vector in the same
+    statement: the lanes of a row's group each store to some of the copies, so
+    a lane may read an entry that another lane has already replaced."""
+    return [m.group(0) for m in re.finditer(r"\b(\w+)\.put\s*\([^;]*?\b\1\.get\s*\([^;]*;", text)]
+
+
+def test_replicated_entries_are_read_before_any_lane_stores():
+    text = sources()
+    assert own_entry_stores(text) == []
+    # a row's own entry is read before the reduction, and the lanes meet between
+    for f, read, store in (("csr_phase", "own(m.q)", "done("), ("gs_sweep_cl", "xi = x.get(i)", ".put(")):
+        body = body_of(text, f, "__device__")
+        assert body.index(read) < body.index("group_reduce") < body.index("__syncwarp()") < \
+            body.index(store), f
+    assert own_entry_stores("auto add = [&](int i) { x.put(i, x.get(i) + s, gl, pG, C); };")
+    assert not own_entry_stores("t.put(i, b.get(i) - s, gl, G, C); x.put(i, o + s, gl, G, C);")
