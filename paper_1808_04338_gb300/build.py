@@ -51,7 +51,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
     nvcc = _nvcc()
     headers = [os.path.join(CSRC, "dp_internal.h"), os.path.join(CSRC, "dp_kernels.cuh"),
-               os.path.join(CSRC, "dp_tma.cuh"), os.path.join(ROOT, "include", "dpsim.h")]
+               os.path.join(CSRC, "dp_tma.cuh"), os.path.join(CSRC, "dp_device.h"),
+               os.path.join(ROOT, "include", "dpsim.h")]
     jobs = []
     objs = []
     for src, extra in UNITS.items():

@@ -708,10 +708,11 @@ int cluster_refresh(Sim *s, bool coarse) {
 }
 
 // Cluster size: 16 CTAs if the GPU can place them, else 8, else 0.  Asked
-// once: the occupancy queries cost more than the rest of cluster_setup, and
-// they serialise the set-ups of several host threads.
+// once on each device: the occupancy queries cost more than the rest of
+// cluster_setup, and they serialise the set-ups of several host threads.
 static int cluster_ctas() {
-  static const int ctas = [] {
+  static PerDevice per;
+  return per([] {
     using Cycle64 = void (*)(const LevelDev<double> *, int, int, const double *, double *,
                              const double *, const int *, const double *, int, int, int);
     using Cycle32 = void (*)(const LevelDev<float> *, int, int, const float *, float *,
@@ -751,8 +752,7 @@ static int cluster_ctas() {
       cudaGetLastError();
     }
     return csize;
-  }();
-  return ctas;
+  });
 }
 
 // Decide the first level run by the cluster kernel and the cluster size; copy

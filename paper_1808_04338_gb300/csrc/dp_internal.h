@@ -8,6 +8,7 @@
 #include <utility>
 #include <vector>
 
+#include "dp_device.h"
 #include "dpsim.h"
 
 namespace dp {

@@ -1408,16 +1408,13 @@ __global__ void __launch_bounds__(64) k_dense_cols(int n, const double *__restri
 }
 
 template <int R>
-static void dense_cols(Sim *s, int n) {
-  static const bool once = [] {
-    cudaFuncSetAttribute(k_dense_cols<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         kFactorMax * kFactorMax * 8);
-    return true;
-  }();
-  (void)once;
+static int dense_cols(Sim *s, int n) {
+  DP_CUDA(s, (kernel_attribute<k_dense_cols<R>, cudaFuncAttributeMaxDynamicSharedMemorySize>(
+                 kFactorMax * kFactorMax * 8)));
   int ldo = factor_ld(n);
   DP_LAUNCH(s, k_dense_cols<R>, nblk(n, 2), 64, (size_t)n * ldo * 8, n, s->coarse_lu, ldo,
             s->coarse_piv, s->coarse_lu + (size_t)n * ldo, s->coarse_inv);
+  return DP_OK;
 }
 
 int coarse_factor(Sim *s) {
@@ -1440,21 +1437,17 @@ int coarse_factor(Sim *s) {
   }
   s->coarse_n = n;
   if (n <= kFactorMax) {
-    static const bool once = [] {
-      cudaFuncSetAttribute(k_dense_factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)factor_smem(kFactorMax));
-      return true;
-    }();
-    (void)once;
+    DP_CUDA(s, (kernel_attribute<k_dense_factor, cudaFuncAttributeMaxDynamicSharedMemorySize>(
+                   (int)factor_smem(kFactorMax))));
     int ldo = factor_ld(n);
     DP_LAUNCH(s, k_dense_factor, 1, kFactorThreads, factor_smem(n), n, L.rowptr, L.col, L.val,
               s->coarse_lu, ldo, s->coarse_piv, s->coarse_lu + (size_t)n * ldo);
     switch ((n + 31) / 32) {
-      case 1: dense_cols<1>(s, n); break;
-      case 2: dense_cols<2>(s, n); break;
-      case 3: dense_cols<3>(s, n); break;
-      case 4: dense_cols<4>(s, n); break;
-      default: dense_cols<5>(s, n); break;
+      case 1: DP_TRY(dense_cols<1>(s, n)); break;
+      case 2: DP_TRY(dense_cols<2>(s, n)); break;
+      case 3: DP_TRY(dense_cols<3>(s, n)); break;
+      case 4: DP_TRY(dense_cols<4>(s, n)); break;
+      default: DP_TRY(dense_cols<5>(s, n)); break;
     }
     DP_CUDA(s, cudaGetLastError());
     return DP_OK;
@@ -1998,19 +1991,26 @@ __global__ void __launch_bounds__(kTT + 32) k_resid_c_tma(int r0, int r1,
   sweep_tma_body<T, true, S, CAPR>(r0, r1, rowptr, colp, pv, nullptr, b, x, r, err);
 }
 
+// CTAs of a pipelined kernel that fit on the current device at once, its
+// dynamic shared memory limit raised first
+template <typename K>
+static int resident_ctas(K kern, int smem) {
+  int dev = 0, nsm = 0, n = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return -(int)e;   // asked again next time; the launch reports it
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kTT + 32, smem);
+  return std::max(n, 1) * std::max(nsm, 1);
+}
+
 // grid of a pipelined kernel: its tiles, at most the CTAs that fit on the
-// GPU at once (queried once per kernel, thread-safe; ID tells the kernels
-// of one signature apart)
+// GPU at once (queried once per kernel and device; ID tells the kernels of
+// one signature apart)
 template <int ID, typename K>
 static int tma_grid(K kern, int smem, int rows) {
-  static const int slots = [&]() {
-    int dev = 0, nsm = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kTT + 32, smem);
-    return std::max(n, 1) * std::max(nsm, 1);
-  }();
+  static PerDevice per;
+  const int slots = per([&] { return resident_ctas(kern, smem); });
   return std::max(1, std::min((rows + kTT - 1) / kTT, slots));
 }
 
@@ -2204,18 +2204,12 @@ static int gs_sweep_persistent(Sim *s, const SweepPlan &plan, const T *pv, const
                                const T *b, T *x) {
   constexpr int smem = S * (int)sizeof(TStage<T, CAPR>);
   auto kern = k_gs_c_sweep<T, S, CAPR>;
-  static const int slots = [&]() {
-    int dev = 0, nsm = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kTT + 32, smem);
-    return std::max(n, 1) * std::max(nsm, 1);
-  }();
+  static PerDevice per;
+  const int slots = per([&] { return resident_ctas(kern, smem); });
   int tiles = 1;
   for (int p = 0; p < plan.nphase; ++p)
     tiles = std::max(tiles, (plan.r1[p] - plan.r0[p] + kTT - 1) / kTT);
-  int grid = std::min(slots, tiles);
+  int grid = std::max(1, std::min(slots, tiles));
   if (s->alloc_failed) return DP_ENOMEM;
   s->waits_used = true;
   LaunchScope ls(s, "k_gs_c_sweep");

@@ -403,11 +403,9 @@ static int launch_cluster(Sim *s, const char *name, K kern, const Args &A) {
 
 template <typename T, int PART>
 static int launch_small(Sim *s, const SmallArgs<T> &A) {
-  static const bool once = [] {   // clusters of 16 CTAs
-    cudaFuncSetAttribute(k_cpr_small<T, PART>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    return true;
-  }();
-  (void)once;
+  // clusters of 16 CTAs
+  DP_CUDA(s, (kernel_attribute<k_cpr_small<T, PART>,
+                               cudaFuncAttributeNonPortableClusterSizeAllowed>(1)));
   return launch_cluster(s, "k_cpr_small", k_cpr_small<T, PART>, A);
 }
 
@@ -627,11 +625,7 @@ int orth_small_step(Sim *s, int j, const double *z, double *vnext) {
   A.z = z; A.V = s->V; A.vnext = vnext;
   A.H = s->H; A.cs = s->cs; A.sn = s->sn; A.g = s->g; A.scal = s->scal;
   A.reorth = s->opt.reorth;
-  static const bool once = [] {
-    cudaFuncSetAttribute(k_orth_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    return true;
-  }();
-  (void)once;
+  DP_CUDA(s, (kernel_attribute<k_orth_small, cudaFuncAttributeNonPortableClusterSizeAllowed>(1)));
   return launch_cluster(s, "k_orth_small", k_orth_small, A);
 }
 
