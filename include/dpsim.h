@@ -352,9 +352,9 @@ int sim_autotune(dp_sim *sim, int32_t reps, char *report, int32_t report_len);
 
 /* Sets the kernel of level 0's Gauss-Seidel colours and residual when level
  * 0 runs in the ILU(0) colour order (what sim_autotune chooses; the default
- * is -1, and 1, with the same results, in a server of several workers or a
- * sim_advance_many of several threads: on a GPU shared by many streams -1 is
- * the slower one):
+ * is -1 for a realisation on the default stream and in a server of one
+ * worker, and 1, with the same results, on a stream of its own: where several
+ * streams' kernels share the GPU -1 is the slower one):
  *    1  a thread per row;
  *    0  a CTA's rows and their entries staged in shared memory first;
  *   -1, -2, -3  a persistent kernel whose producer warp brings tiles of

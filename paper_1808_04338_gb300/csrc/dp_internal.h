@@ -404,11 +404,11 @@ struct Sim {
   float *p0c_valf = nullptr, *dinv_cf = nullptr;
   bool l0_lu = false;
   // the kernel of the level-0 colour-order sweeps and residual
-  // (sim_set_l0_kernel): the pipelined one was the fastest or within 2% of it
-  // from 5765 rows (two sweeps and a residual 12.5 us, a thread per row 15.5)
-  // to 4M (128 and 155), in FP64 too (200005 rows: 32.7 and 45.2)
+  // (sim_set_l0_kernel; the default: l0_default).  Alone on the GPU the
+  // pipelined one (-1) was the fastest or within 2% of it from 5765 rows (two
+  // sweeps and a residual 12.5 us, a thread per row 15.5) to 4M (128 and 155),
+  // in FP64 too (200005 rows: 32.7 and 45.2)
   int l0_G = -1;
-  bool l0_chosen = false;   // by sim_set_l0_kernel or sim_autotune: see l0_share
   int shapes = 0;     // bumped whenever launch shapes change (autotune, AMG set-up)
   double *l0_pv = nullptr;
   float *l0_pvf = nullptr;   // inverse from the LU factors (n <= kInverseMax), row-major

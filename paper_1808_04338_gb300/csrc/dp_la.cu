@@ -2602,7 +2602,6 @@ static int tune_l0(Sim *s, int reps, std::string &rep) {
     if (ms < best_ms) { best_ms = ms; best = g; }
   }
   s->l0_G = best;
-  s->l0_chosen = true;
   std::snprintf(buf, sizeof buf, "level 0 colour sweeps and residual lanes %d -> %d (us per two sweeps+residual:%s)\n",
                 old, best, line.c_str());
   rep += buf;

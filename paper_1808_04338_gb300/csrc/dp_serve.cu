@@ -178,8 +178,8 @@ void dp_server::worker() {
         r.rock.phi_f = r.phi_f.data(); r.rock.phi_m = r.phi_m.data();
         rc = sim_create(&r.grid, &r.rock, &r.fluid, r.wells.data(), (int32_t)r.wells.size(),
                         &opts, nullptr, (void *)r.stream, &r.sim);
-        // the level-0 kernel for a GPU that several streams share
-        if (rc == DP_OK && several) rc = sim_set_l0_kernel(r.sim, 1);
+        // one request at a time: the level-0 kernel of a GPU that no other stream uses
+        if (rc == DP_OK && !several) rc = sim_set_l0_kernel(r.sim, -1);
         if (rc == DP_OK) rc = sim_set_state(r.sim, r.p.data(), r.sw.data(), r.bhp.data());
       }
     }

@@ -186,6 +186,20 @@ static bool bad_opts(const dp_options *o) {
          o->schur < 0 || o->schur > 1 || !(o->reorth >= 0.0) || !std::isfinite(o->reorth);
 }
 
+// Level 0's kernel until sim_set_l0_kernel or sim_autotune chooses one (the
+// results are the same bit for bit): the pipelined one on the default stream,
+// a thread per row on a stream of its own.  The pipelined kernel is the faster
+// one alone, but its CTAs hold their SMs for a whole colour and wait for
+// shared memory that other streams' kernels hold, and a realisation is given
+// its own stream to overlap with others.  A timestep of 1, 4, 8 and 16
+// realisations, a host thread and a stream each, pipelined and a thread per
+// row (ms a timestep): 25k rows 5.32 and 5.57, 1.77 and 1.81, 1.26 and
+// 1.27, 0.95 and 0.95; 196k rows 8.56 and 8.81, 4.38 and 4.23, 3.77 and
+// 3.41, 3.61 and 3.11; 1M rows (to 8) 24.2 and 24.7, 21.5 and 18.8, 21.9 and 18.0.
+static int l0_default(cudaStream_t stream) {
+  return stream == nullptr || stream == cudaStreamLegacy ? -1 : 1;
+}
+
 extern "C" int sim_create(const dp_grid *grid, const dp_rock *rock, const dp_fluid *fluid,
                           const dp_well *wells, int32_t nwells, const dp_options *opts,
                           const dp_allocator *alloc, void *stream, dp_sim **out) {
@@ -219,6 +233,7 @@ extern "C" int sim_create(const dp_grid *grid, const dp_rock *rock, const dp_flu
   if (!s) return DP_ENOMEM;
   s->opt = *opts;
   s->stream = (cudaStream_t)stream;
+  s->l0_G = l0_default(s->stream);
   if (alloc && alloc->alloc && alloc->free) { s->alloc = *alloc; s->own_alloc = false; }
   else { s->alloc.alloc = default_alloc; s->alloc.free = default_free; s->alloc.ctx = nullptr; }
   s->wells.assign(wells, wells + nwells);
@@ -662,24 +677,10 @@ extern "C" int sim_solver_sizes(dp_sim *s, int32_t *nb, int32_t *nnzb) {
   return DP_OK;
 }
 
-// Realisations that share the GPU with others, each on its own stream, take
-// level 0's thread-per-row kernel by default: the pipelined kernel's CTAs hold
-// their SMs for a whole colour and wait for shared memory that other streams'
-// hold.  A stream of 512 requests on 16 workers, 128 realisations: cold p50
-// 126 ms with it and 205 with the pipelined one, warm 18.3 and 30.7 ms (the
-// same results bit for bit).
-static void l0_share(Sim *s) {
-  if (s->l0_chosen || s->l0_G == 1) return;
-  s->l0_G = 1;
-  graphs_free(s);
-  ++s->shapes;
-}
-
 extern "C" int sim_set_l0_kernel(dp_sim *s, int32_t variant) {
   if (!s || variant < -4 || variant > 8 || (variant > 2 && variant != 4 && variant != 8))
     return DP_EINVAL;
   DP_TRY(unusable(s));
-  s->l0_chosen = true;
   if (s->l0_G != variant) {
     s->l0_G = variant;
     graphs_free(s);   // the Arnoldi steps are captured again
@@ -719,8 +720,6 @@ extern "C" int sim_advance_many(dp_sim *const *sims, int32_t n, const double *dt
   }
   int nt = threads > 0 ? threads : std::min<int>(n, 16);
   nt = std::max(1, std::min(nt, n));
-  if (nt > 1)
-    for (int k = 0; k < n; ++k) l0_share(sims[k]);
   std::vector<int> rc(n, DP_OK);
   std::atomic<int> next{0};
   auto worker = [&]() {
