@@ -1042,6 +1042,9 @@ int lanes_for(double mean_len) {
 // 2.4 on the last instead of 3.6 at 16), restriction 2, 8, 16, 16 (2.4 us into
 // the third instead of 3.9 at 4); FP64 on 144677, 22225, 3411 rows: operator
 // 2, 4, 16 (17.4, 9.0 and 4.5 us; with 4, 8 and 16 21.7, 10.9 and 4.5).
+// The FP32 operator's last two lines: lanes that would have fewer than 1.25
+// entries each are halved, and a launch of at most 8192 threads, which leaves
+// most of the GPU idle, takes up to a lane an entry.
 int cycle_lanes(int op, bool f64, double rows, double len) {
   double per = f64 ? (op == 0 || op == 2 ? 2.0 : 1.0) : (op == 0 ? 1.6 : 1.0);
   double cap = f64 ? (op == 2 ? 6.0e4 : 9.0e4) : (op == 0 ? 2.5e6 : op == 1 ? 1.2e6 : 2.0e5);

@@ -412,7 +412,13 @@ static int launch_small(Sim *s, const SmallArgs<T> &A) {
 // The sizes where the cluster launches beat the launches of a phase each:
 // its 16 SMs are 10-20% faster over a timestep up to 7845 rows, equal from
 // 11565 (FP32 7.8 and 7.8 ms, FP64 65.4 and 66.9) and slower at 33125 (FP32
-// 8.4 against 6.8 ms).  cluster_rows < 0 asks for no cluster launch.
+// 8.4 against 6.8 ms).  With other streams on the GPU too: 1, 4, 8 and 16
+// realisations, a thread and a stream each, cluster launches and a launch a
+// phase (ms a timestep): 602 rows FP64 18.0 and 20.7, 4.99 and 5.99, 3.15 and
+// 3.59, 2.14 and 2.24, FP32 3.73 and 4.00, 1.27 and 1.30, 1.07 and 1.05, 1.07
+// and 1.04; 8002 rows FP64 47.2 and 48.4, 12.3 and 13.7, 8.51 and 9.95, 7.11
+// and 7.92, FP32 4.59 and 4.64, 1.56 and 1.63, 1.07 and 1.12, 0.92 and 0.94.
+// cluster_rows < 0 asks for no cluster launch.
 constexpr int kSmallRows = 8192;
 
 bool cpr_small(const Sim *s) {

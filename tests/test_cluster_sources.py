@@ -5,7 +5,7 @@ known to have started: a kernel that does has arrived at and waited for a
 cluster barrier before its first such access."""
 import re
 
-from test_pdl_sources import body_of, sources
+from test_pdl_sources import body_of, sources, stores
 
 REMOTE = re.compile(r"map_shared_rank\s*\(|\bmapa\.")
 BARRIER = re.compile(r"\bcl\.sync\(\)|\b(?:cl|small)_wait\(\)|barrier_wait\s*\(")
@@ -73,3 +73,16 @@ def test_replicated_entries_are_read_before_any_lane_stores():
             body.index(store), f
     assert own_entry_stores("auto add = [&](int i) { x.put(i, x.get(i) + s, gl, pG, C); };")
     assert not own_entry_stores("t.put(i, b.get(i) - s, gl, G, C); x.put(i, o + s, gl, G, C);")
+
+
+def test_cluster_kernels_launched_as_dependents_wait_before_they_store():
+    """The kernels launched through cudaLaunchKernelEx as programmatic
+    dependents, which the check of DP_LAUNCH_PDL's kernels does not see: they
+    reach griddep_wait before any store, and let their own dependents in only
+    after it."""
+    text = sources()
+    for k in ("k_coarse_cycle", "k_cpr_small", "k_orth_small"):
+        body = body_of(text, k, "__global__")
+        wait = body.index("griddep_wait()")
+        assert wait < body.index("griddep_launch_dependents()"), k
+        assert stores(body[:wait]) == [], k
