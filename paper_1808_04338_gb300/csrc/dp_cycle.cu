@@ -688,14 +688,14 @@ static int ell_build(Sim *s, Level &L) {
 
 // Copy the current level values into the padded copies when the hierarchy's
 // values have been refreshed (with their FP32 copies); otherwise (coarse =
-// false) only level 0's are new, which are the pressure block itself.
+// false) only level 0's 1/a_ii is new.
 int cluster_refresh(Sim *s, bool coarse) {
   if (s->cl_level < 0) return DP_OK;
   bool f32 = s->opt.precision >= 1;
   for (int l = s->cl_level; l < (int)s->lev.size() && (coarse || l == 0); ++l) {
     Level &L = s->lev[l];
     if (!L.ell_src) continue;
-    const long long total = L.ell_total;
+    long long total = coarse ? L.ell_total : 0;
     if (f32)
       DP_LAUNCH(s, k_ell_values<float>, nblk(total + L.n), kBlock, 0, total, L.ell_src, L.valf,
                 L.ell_valf, L.n, L.clist, L.dinvf, L.ell_dinvf);
