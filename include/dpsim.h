@@ -147,8 +147,10 @@ typedef struct {
                             uses Gauss-Seidel, else never */
   int32_t amg_refresh;   /* 0: the prolongators and coarse operators are recomputed
                             every Newton iteration; 1: only at the first Newton
-                            iteration of a timestep (level 0, the pressure block,
-                            always takes the current values) */
+                            iteration of a timestep; level 0, the pressure block,
+                            takes the current values, except inside the cluster
+                            kernel, whose sweeps keep its entries of that first
+                            iteration too (1/a_ii current in FP64) */
   int32_t decouple;      /* D of Eq. "decoupled-eq", per cell block row (well rows
                             unchanged): 0 the modified Gauss-Jordan step, read as
                             the elimination of the pressure row's saturation

@@ -688,7 +688,11 @@ static int ell_build(Sim *s, Level &L) {
 
 // Copy the current level values into the padded copies when the hierarchy's
 // values have been refreshed (with their FP32 copies); otherwise (coarse =
-// false) only level 0's 1/a_ii is new.
+// false) only level 0's 1/a_ii, in FP64: its sweeps keep the entries of the
+// last refresh, and in FP32 all of level 0 is of that refresh (mixed_refresh).
+// With the current entries a timestep took as many iterations (0.7% fewer over
+// 400 timesteps of 11k and 16k rows) and one in sixteen ended more than the
+// Newton tolerance away from the state it ends in so.
 int cluster_refresh(Sim *s, bool coarse) {
   if (s->cl_level < 0) return DP_OK;
   bool f32 = s->opt.precision >= 1;

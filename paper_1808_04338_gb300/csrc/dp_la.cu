@@ -3105,7 +3105,8 @@ int mixed_refresh(Sim *s, bool coarse) {
   for (size_t l = 0; l < s->lev.size(); ++l) {
     if (!coarse) {
       // level 0 only; in colour order its FP32 values and 1/a_ii come from the
-      // decoupling and from l0_refresh instead
+      // decoupling and from l0_refresh instead (the cluster cycle, when it
+      // takes level 0, keeps those of the last refresh)
       Level &L = s->lev[0];
       if (!s->l0c) {
         DP_LAUNCH(s, k_to_f32_i, nblk(L.nnz), kBlock, 0, (long long)L.nnz, L.val, L.valf);
