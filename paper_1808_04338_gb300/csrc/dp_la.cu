@@ -1271,10 +1271,9 @@ __global__ void k_dense_inverse(int n, const double *a, const int *piv, double *
 // step.  An FP64 instruction holds a quarter of the SM for 64 cycles, so the
 // pivot warp shares its quarter with no updating warp and divides once a
 // step.  The multipliers, and the entries of the inverse's columns, are
-// quotients by the pivot's reciprocal and a correction (quotient), a lane's
-// side by side: 97 rows 262 us, the columns 49 us (one after another 294 and
-// 54; 128 rows 368 and 62, 354 and 67); with the division 505 and 105 us, with
-// the product alone, which rounds twice, 232 and 39 us (over the coarsest
+// quotients by the pivot's reciprocal and a correction (quotient): 97 rows
+// 294 us, the columns 55 us; with the division 505 and 105 us, with the
+// product alone, which rounds twice, 232 and 39 us (over the coarsest
 // operators of sixteen synthetic models the inverse's error against 64 bits
 // was 1.03 times that of quotients in the mean).  Output: lu column-major in
 // pivot order (leading dimension ldo, even, so that the columns can be read as
@@ -1283,46 +1282,6 @@ __global__ void k_dense_inverse(int n, const double *a, const int *piv, double *
 constexpr int kFactorMax = 160, kFactorThreads = 512;
 inline int factor_ld(int n) { return (n + 1) & ~1; }
 inline size_t factor_smem(int n) { return ((size_t)n * (n | 1) + 2 * (size_t)n) * 8; }
-
-// A column's multipliers by one warp (R = ceil(n / 32) rows a lane, their
-// quotients side by side): rows without a pivot yet, into the column (stride
-// ld) and m.
-template <int R>
-__device__ __forceinline__ void dense_multipliers(int n, double *col, int ld, const int *order,
-                                                  double d, double r, double *m, int lane) {
-  double a[R], l[R];
-  bool in[R], all = true;
-#pragma unroll
-  for (int c = 0; c < R; ++c) {
-    const int i = lane + 32 * c;
-    in[c] = i < n && order[i] == n;
-    a[c] = in[c] ? col[i * ld] : 0.0;
-  }
-#pragma unroll
-  for (int c = 0; c < R; ++c) {
-    bool ok;
-    l[c] = quotient_if(a[c], d, r, &ok);
-    all = all && ok;
-  }
-  if (!all) {
-#pragma unroll 1
-    for (int c = 0; c < R; ++c) {
-      const int i = lane + 32 * c;
-      if (i < n && order[i] == n) {
-        const double v = quotient(col[i * ld], d, r);
-        col[i * ld] = v;
-        m[i] = v;
-      }
-    }
-    return;
-  }
-#pragma unroll
-  for (int c = 0; c < R; ++c)
-    if (in[c]) {
-      col[(lane + 32 * c) * ld] = l[c];
-      m[lane + 32 * c] = l[c];
-    }
-}
 
 __global__ void __launch_bounds__(kFactorThreads) k_dense_factor(int n, const int *rowptr,
                                                                  const int *col,
@@ -1366,14 +1325,12 @@ __global__ void __launch_bounds__(kFactorThreads) k_dense_factor(int n, const in
       rdiag[k] = r;
     }
     __syncwarp();
-    double *m = mult + (k & 1) * n;
-    switch ((n + 31) >> 5) {
-      case 1: dense_multipliers<1>(n, A + k, ld, order, d, r, m, lane); break;
-      case 2: dense_multipliers<2>(n, A + k, ld, order, d, r, m, lane); break;
-      case 3: dense_multipliers<3>(n, A + k, ld, order, d, r, m, lane); break;
-      case 4: dense_multipliers<4>(n, A + k, ld, order, d, r, m, lane); break;
-      default: dense_multipliers<5>(n, A + k, ld, order, d, r, m, lane); break;
-    }
+    for (int i = lane; i < n; i += 32)
+      if (order[i] == n) {
+        double l = quotient(A[i * ld + k], d, r);
+        A[i * ld + k] = l;
+        mult[(k & 1) * n + i] = l;
+      }
     __syncwarp();
   };
   if (warp == 0) panel(0);
@@ -1420,8 +1377,8 @@ __global__ void __launch_bounds__(64) k_dense_cols(int n, const double *__restri
   for (int r = 0; r < R; ++r) {
     int i = lane + 32 * r;
     x[r] = i < n && __ldg(prow + i) == c ? 1.0 : 0.0;
-    d[r] = i < n ? fac[(size_t)i * ldo + i] : 1.0;   // past the end: 0 by 1
-    rd[r] = i < n ? __ldg(rdiag + i) : 1.0;
+    d[r] = i < n ? fac[(size_t)i * ldo + i] : 0.0;
+    rd[r] = i < n ? __ldg(rdiag + i) : 0.0;
   }
 #pragma unroll
   for (int b = 0; b < R; ++b)

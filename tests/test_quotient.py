@@ -57,7 +57,6 @@ def test_quotients_are_those_of_the_division(tmp_path):
 
 def test_the_dense_factorisation_forms_quotients():
     text = sources()
-    assert "dense_multipliers<" in body_of(text, "k_dense_factor", "__global__")
-    for name, kind in (("dense_multipliers", "__device__"), ("k_dense_cols", "__global__")):
-        body = body_of(text, name, kind)
-        assert "quotient(" in body and "] * r;" not in body and "* rd[" not in body, name
+    for kernel in ("k_dense_factor", "k_dense_cols"):
+        body = body_of(text, kernel, "__global__")
+        assert "quotient(" in body and "] * r;" not in body and "* rd[" not in body, kernel
