@@ -52,6 +52,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     nvcc = _nvcc()
     headers = [os.path.join(CSRC, "dp_internal.h"), os.path.join(CSRC, "dp_kernels.cuh"),
                os.path.join(CSRC, "dp_tma.cuh"), os.path.join(CSRC, "dp_device.h"),
+               os.path.join(CSRC, "dp_quotient.h"),
                os.path.join(ROOT, "include", "dpsim.h")]
     jobs = []
     objs = []

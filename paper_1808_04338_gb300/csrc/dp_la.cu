@@ -10,6 +10,7 @@
 
 #include "dp_internal.h"
 #include "dp_kernels.cuh"
+#include "dp_quotient.h"
 #include "dp_tma.cuh"
 
 namespace dp {
@@ -1270,10 +1271,11 @@ __global__ void k_dense_inverse(int n, const double *a, const int *piv, double *
 // step.  An FP64 instruction holds a quarter of the SM for 64 cycles, so the
 // pivot warp shares its quarter with no updating warp and divides once a
 // step (97 rows: 474 us with a division a multiplier and every warp
-// updating, 229 us so).  Output: lu column-major in pivot order (leading dimension ldo, even,
-// so that the columns can be read as 16-byte words), prow[k] the row of
-// pivot k, rdiag[k] its reciprocal (0 for a zero pivot, whose multipliers
-// are then 0 as well).
+// updating, 232 us so; the multipliers and the entries of the inverse's
+// columns round twice, see quotient).  Output: lu column-major in pivot order
+// (leading dimension ldo, even, so that the columns can be read as 16-byte
+// words), prow[k] the row of pivot k, rdiag[k] its reciprocal (0 for a zero
+// pivot, whose multipliers are then 0 as well).
 constexpr int kFactorMax = 160, kFactorThreads = 512;
 inline int factor_ld(int n) { return (n + 1) & ~1; }
 inline size_t factor_smem(int n) { return ((size_t)n * (n | 1) + 2 * (size_t)n) * 8; }
@@ -1322,7 +1324,7 @@ __global__ void __launch_bounds__(kFactorThreads) k_dense_factor(int n, const in
     __syncwarp();
     for (int i = lane; i < n; i += 32)
       if (order[i] == n) {
-        double l = A[i * ld + k] * r;
+        double l = quotient(A[i * ld + k], d, r);
         A[i * ld + k] = l;
         mult[(k & 1) * n + i] = l;
       }
@@ -1367,12 +1369,13 @@ __global__ void __launch_bounds__(64) k_dense_cols(int n, const double *__restri
   __syncthreads();
   const int lane = threadIdx.x & 31, c = 2 * blockIdx.x + (threadIdx.x >> 5);
   if (c >= n) return;   // whole warps
-  double x[R], rd[R];
+  double x[R], d[R], rd[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     int i = lane + 32 * r;
     x[r] = i < n && __ldg(prow + i) == c ? 1.0 : 0.0;
-    rd[r] = i < n ? __ldg(rdiag + i) : 0.0;
+    d[r] = i < n ? fac[(size_t)i * ldo + i] : 1.0;   // past the end: 0 by 1
+    rd[r] = i < n ? __ldg(rdiag + i) : 1.0;
   }
 #pragma unroll
   for (int b = 0; b < R; ++b)
@@ -1394,7 +1397,7 @@ __global__ void __launch_bounds__(64) k_dense_cols(int n, const double *__restri
     for (int kk = 31; kk >= 0; --kk) {
       int k = 32 * b + kk;
       if (k >= n) continue;
-      double xk = __shfl_sync(0xffffffffu, x[b] * rd[b], kk);
+      double xk = __shfl_sync(0xffffffffu, quotient(x[b], d[b], rd[b]), kk);
       if (lane == kk) x[b] = xk;
       const double *u = fac + (size_t)k * ldo;
 #pragma unroll
